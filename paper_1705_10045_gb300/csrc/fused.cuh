@@ -35,9 +35,7 @@
 // (c_{k+1} = -c_k), which share the even part of every term.
 #pragma once
 
-#include <type_traits>
-
-#include "kernels.cuh"
+#include "node.cuh"
 
 namespace lbm {
 
@@ -85,20 +83,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity
     } while (clock64() - t0 < 1000000000ll);
     return false;
 }
-
-// Velocity of direction k in march coordinates: (a, b) across the tile,
-// m along the march axis.
-template <int Q> struct MVel;
-template <> struct MVel<9> {
-    __host__ __device__ static constexpr int a(int k) { return Vel<9>::cx(k); }
-    __host__ __device__ static constexpr int b(int) { return 0; }
-    __host__ __device__ static constexpr int m(int k) { return Vel<9>::cy(k); }
-};
-template <> struct MVel<19> {
-    __host__ __device__ static constexpr int a(int k) { return Vel<19>::cx(k); }
-    __host__ __device__ static constexpr int b(int k) { return Vel<19>::cy(k); }
-    __host__ __device__ static constexpr int m(int k) { return Vel<19>::cz(k); }
-};
 
 // Geometry of the march: na x nb tile plane (nb = 1 for D2Q9), nm planes.
 struct MarchGeom {
