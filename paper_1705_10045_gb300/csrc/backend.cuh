@@ -359,12 +359,14 @@ template <int Q, typename S, typename R> struct Impl {
     static int batch_build(lbm_batch* b);
     static int batch_launch(lbm_batch* b, int advance);
 
-    static int reduce(lbm_handle* h, double* out_dev) {
+    // sums over nodes [i0, i0 + n) and the device counters: 8 doubles at out_dev
+    static int reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev) {
         const KParams<R> kp = make_kparams<R>(h);
-        reduce_kernel<Q, S, R><<<kReduceBlocks, kReduceThreads, 0, h->stream>>>((const S*)h->pop[h->cur], kp,
-                                                                                h->partials);
-        reduce_final_kernel<<<1, 32, 0, h->stream>>>(h->partials, kReduceBlocks, out_dev);
-        return cuda_error(cudaGetLastError(), "lbm_diagnostics launch");
+        const int blocks = reduce_blocks(n);
+        reduce_kernel<Q, S, R><<<blocks, kReduceThreads, 0, h->stream>>>((const S*)h->pop[h->cur], h->nn, i0, n, kp,
+                                                                         partials);
+        reduce_final_kernel<<<kSums, 32, 0, h->stream>>>(partials, blocks, out_dev, (const Counters*)h->cnt);
+        return cuda_error(cudaGetLastError(), "conservation sums launch");
     }
 };
 
@@ -427,7 +429,9 @@ template <int Q> int Backend<Q>::init(lbm_handle* h, const double* rho, const do
 template <int Q> int Backend<Q>::moments(lbm_handle* h, double* rho, double* u, double* T, double* P) {
     LBM_DISPATCH(h, moments(h, rho, u, T, P));
 }
-template <int Q> int Backend<Q>::reduce(lbm_handle* h, double* out_dev) { LBM_DISPATCH(h, reduce(h, out_dev)); }
+template <int Q> int Backend<Q>::reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev) {
+    LBM_DISPATCH(h, reduce(h, i0, n, partials, out_dev));
+}
 #define LBM_BATCH_DISPATCH(b, CALL)                                              \
     switch ((b)->common.storage) {                                               \
         case LBM_STORE_FP64: return Impl<Q, double, double>::CALL;               \

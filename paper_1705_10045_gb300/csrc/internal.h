@@ -78,6 +78,10 @@ struct TraceRange {
 void set_error(const std::string& msg);
 int cuda_error(cudaError_t e, const char* where);
 int ensure_staging(lbm_handle* h);   // the handle's host-transfer buffer, allocated on first use
+// Conservation sums of nodes [i0, i0 + n) through `partials` (block partials,
+// then 8 results): out[0..4] the sums, out[5] clamped and out[6] bad nodes.
+// Synchronising; returns a latched device error if any.
+int diagnose(lbm_handle* h, long long i0, long long n, double* partials, double out[8]);
 
 
 // per-lattice entry points, dispatched on the storage format inside
@@ -89,7 +93,8 @@ template <int Q> struct Backend {
     static int launches(const lbm_handle* h);
     static int init(lbm_handle* h, const double* rho, const double* u, const double* eps);   // device pointers
     static int moments(lbm_handle* h, double* rho, double* u, double* T, double* P);       // device pointers
-    static int reduce(lbm_handle* h, double* out_dev);   // 5 sums into device memory
+    // sums over nodes [i0, i0 + n): 5 sums and 3 counters into device memory
+    static int reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev);
     static size_t field_bytes(int storage);
     // batches: shapes, work table, descriptors, and one request (clear, the
     // persistent launch, and the descriptor advance when `advance`)

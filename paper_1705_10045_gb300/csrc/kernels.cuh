@@ -280,25 +280,24 @@ __global__ void __launch_bounds__(256) output_kernel(const R* __restrict__ fld, 
 
 // ---------------------------------------------------------------------------
 // Conservation sums in FP64 with Kahan compensation.  Each thread walks a
-// fixed strided set of nodes, blocks combine in a fixed shuffle tree and a
-// single block sums the block partials in index order: bitwise reproducible
-// for a fixed grid.
+// fixed strided set of nodes, blocks combine in a fixed shuffle tree and one
+// more block sums the block partials in a fixed order: bitwise reproducible
+// for a given number of nodes.
 
-constexpr int kReduceBlocks = 1024;
+constexpr int kReduceBlocks = 1024;   // most blocks (and block partials) of a reduction
 constexpr int kReduceThreads = 256;
 constexpr int kSums = 5;   // mass, momentum x, y, z, energy
 
-// compensated (Kahan) summation in type T; the sum is s - c
-template <typename T> struct KahanT {
-    T s = T(0), c = T(0);
-    __device__ void add(T v) {
-        T y = v - c;
-        T t = s + y;
+// compensated (Kahan) summation; the sum is s - c
+struct Kahan {
+    double s = 0.0, c = 0.0;
+    __device__ void add(double v) {
+        double y = v - c;
+        double t = s + y;
         c = (t - s) - y;
         s = t;
     }
 };
-using Kahan = KahanT<double>;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -306,25 +305,57 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// PAIRS: populations in the library's pair layout; false: set-major planes
-// (a checkpoint buffer, lbm_conservation_sums_noalloc)
+// FP32 to FP64 in integer instructions for normal values (the conversion
+// instruction runs at the FP64 rate: two lanes per clock and SM)
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v);
+    if ((b & 0x7f800000u) - 0x00800000u >= 0x7f000000u) return (double)v;   // zero, subnormal, infinite, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// Blocks of a reduction over n nodes: at least four nodes per thread, so that
+// the FP64 block tails stay a minority, and at most one wave of three blocks
+// per SM (934 us on the pool-boiling domain; four 945, five 997, six 1024).
+constexpr int kReduceCtas = 3;
+inline int reduce_blocks(long long n) {
+    const long long per = 4 * kReduceThreads, b = (n + per - 1) / per, most = 152 * kReduceCtas;
+    return (int)(b < 1 ? 1 : (b > most ? most : b));
+}
+
+// Partial sums of the moments of nodes [i0, i0 + n) of a population buffer
+// whose arrays are nn nodes apart.  PAIRS: the library's pair layout; false:
+// set-major planes (a checkpoint buffer, lbm_conservation_sums_noalloc).
+//
+// Bound by the FP64 pipe before memory: five Kahan additions a node are 20
+// FP64 instructions, at two lanes per clock and SM 1.3 ms for 37.7 M nodes,
+// where the populations stream in 0.85 ms.  So moments formed in FP32 are
+// first added up over kGroup nodes in plain FP64 (exact unless their
+// magnitudes spread over 2^26: 24-bit values in a 53-bit sum) and the group
+// sum enters the compensated one: 7.5 FP64 instructions a node.  FP64 moments
+// enter one by one.  Whole diagnostics call, before -> now: 384 x 384 x 256
+// D3Q19 FP32 2326 -> 934 us, FP16 2128 -> 912, 8192 x 4608 D2Q9 1760 -> 737,
+// 512 x 512 234 -> 48.
 template <int Q, typename S, typename R, bool PAIRS = true>
-__global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const S* __restrict__ pop, KParams<R> p,
+__global__ void __launch_bounds__(kReduceThreads, kReduceCtas) reduce_kernel(const S* __restrict__ pop, long long nn, long long i0,
+                                                                long long n, KParams<R> p,
                                                                 double* __restrict__ partials) {
-    // Each thread sums the moments of its nodes (about nn / 262144 of them,
-    // each formed in the arithmetic type as the step forms it) in FP64 with
-    // Kahan compensation; the partials are combined in FP64 from here on, in
-    // a fixed order, so the sums are FP64 and bitwise reproducible.
+    constexpr int kGroup = sizeof(R) == 4 ? 8 : 1;
     Kahan acc[kSums];
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.nn; i += stride) {
-        R rho, jx, jy, jz, E;
-        node_moments<Q, S, R, PAIRS>(pop, p.nn, i, p, rho, jx, jy, jz, E);
-        acc[0].add((double)rho);
-        acc[1].add((double)jx);
-        acc[2].add((double)jy);
-        acc[3].add((double)jz);
-        acc[4].add((double)E);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kGroup * stride) {
+        double g[kSums];
+#pragma unroll 1
+        for (int j = 0; j < kGroup; ++j) {
+            const long long at = i + j * stride;
+            if (at >= n) break;
+            R m[kSums];
+            node_moments<Q, S, R, PAIRS>(pop, nn, i0 + at, p, m[0], m[1], m[2], m[3], m[4]);
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) g[q] = j == 0 ? widen(m[q]) : g[q] + widen(m[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < kSums; ++q) acc[q].add(g[q]);
     }
     __shared__ double sh[kSums][kReduceThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -341,12 +372,30 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const S* __restr
     }
 }
 
-static __global__ void __launch_bounds__(32) reduce_final_kernel(const double* __restrict__ partials, int nblocks,
-                                                          double* __restrict__ out) {
-    if (threadIdx.x < kSums) {
-        Kahan b;
-        for (int j = 0; j < nblocks; ++j) b.add(partials[(size_t)threadIdx.x * nblocks + j]);
-        out[threadIdx.x] = b.s;
+// The block partials, one block of a warp per sum: Kahan sums per lane, then a tree whose
+// additions carry their rounding errors along.  With cnt, out[5..7] become
+// the clamp, bad-node and timeout counters, so that one copy brings sums and
+// counters to the host.  (One lane per sum over all 1024 partials took 162 us:
+// a chain of 4096 dependent FP64 additions.)
+static __global__ void __launch_bounds__(32) reduce_final_kernel(const double* __restrict__ partials,
+                                                                         int nblocks, double* __restrict__ out,
+                                                                         const Counters* cnt) {
+    const int q = blockIdx.x, lane = threadIdx.x;
+    Kahan b;
+    for (int j = lane; j < nblocks; j += 32) b.add(partials[(size_t)q * nblocks + j]);
+    double s = b.s, e = -b.c;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+        const double t = s + s2, w = t - s;
+        e += e2 + ((s - (t - w)) + (s2 - w));
+        s = t;
+    }
+    if (lane == 0) out[q] = s + e;
+    if (cnt && q == 0 && lane == 0) {
+        out[kSums] = (double)cnt->clamps;
+        out[kSums + 1] = (double)cnt->bad;
+        out[kSums + 2] = (double)cnt->timeouts;
     }
 }
 

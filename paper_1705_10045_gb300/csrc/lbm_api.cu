@@ -142,14 +142,28 @@ int be_init(lbm_handle* h, const double* r, const double* u, const double* e) {
 int be_moments(lbm_handle* h, double* r, double* u, double* T, double* P) {
     return h->Q == 9 ? lbm::Backend<9>::moments(h, r, u, T, P) : lbm::Backend<19>::moments(h, r, u, T, P);
 }
-int be_reduce(lbm_handle* h, double* out) {
-    return h->Q == 9 ? lbm::Backend<9>::reduce(h, out) : lbm::Backend<19>::reduce(h, out);
-}
 
 // FP64 -> FP32, round to nearest (the FP32 twin of the moments)
 __global__ void narrow_kernel(const double* __restrict__ src, float* __restrict__ dst, long long n) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         dst[i] = (float)src[i];
+}
+
+// Report what the device counters say since the last report.
+int latch(lbm_handle* h, unsigned long long bad, unsigned long long timeouts) {
+    if (timeouts) {
+        set_error("fused step: a bounded wait gave up (a producer/consumer hand-off inside a CTA, or in a batch the "
+                  "wait for the domain's previous step; " + std::to_string(timeouts) +
+                  " times); the state is not valid until lbm_init or lbm_set_state");
+        return LBM_ERR_TIMEOUT;
+    }
+    if (bad > h->reported_bad) {
+        h->reported_bad = bad;
+        set_error("non-physical state: non-finite or non-positive density or energy at " + std::to_string(bad) +
+                  " node-steps");
+        return LBM_ERR_NONPHYSICAL;
+    }
+    return LBM_OK;
 }
 
 // Wait for the stream and report non-physical nodes counted since the last report.
@@ -159,22 +173,23 @@ int sync_and_latch(lbm_handle* h) {
     if (rc) return rc;
     rc = cuda_error(cudaStreamSynchronize(h->stream), "stream synchronize");
     if (rc) return rc;
-    if (c.timeouts) {
-        set_error("fused step: a bounded wait gave up (a producer/consumer hand-off inside a CTA, or in a batch the "
-                  "wait for the domain's previous step; " + std::to_string(c.timeouts) +
-                  " times); the state is not valid until lbm_init or lbm_set_state");
-        return LBM_ERR_TIMEOUT;
-    }
-    if (c.bad > h->reported_bad) {
-        h->reported_bad = c.bad;
-        set_error("non-physical state: non-finite or non-positive density or energy at " + std::to_string(c.bad) +
-                  " node-steps");
-        return LBM_ERR_NONPHYSICAL;
-    }
-    return LBM_OK;
+    return latch(h, c.bad, c.timeouts);
 }
 
 }  // namespace
+
+int lbm::diagnose(lbm_handle* h, long long i0, long long n, double* partials, double out[8]) {
+    double* res = partials + kSums * kReduceBlocks;
+    int rc = h->Q == 9 ? Backend<9>::reduce(h, i0, n, partials, res) : Backend<19>::reduce(h, i0, n, partials, res);
+    if (rc) return rc;
+    double got[kSums + 3];
+    rc = cuda_error(cudaMemcpyAsync(got, res, sizeof(got), cudaMemcpyDeviceToHost, h->stream), "sums copy");
+    if (!rc) rc = cuda_error(cudaStreamSynchronize(h->stream), "stream synchronize");
+    if (rc) return rc;
+    rc = latch(h, (unsigned long long)got[kSums + 1], (unsigned long long)got[kSums + 2]);
+    for (int q = 0; q < kSums + 2; ++q) out[q] = got[q];
+    return rc;
+}
 
 extern "C" {
 
@@ -474,19 +489,10 @@ int lbm_diagnostics(lbm_handle* h, double out[8]) {
         return LBM_ERR_INVALID_ARG;
     }
     DeviceGuard dg(h->p.device);
-    double* res = h->partials + lbm::kSums * lbm::kReduceBlocks;
-    int rc;
-    if ((rc = be_reduce(h, res))) return rc;
-    double sums[lbm::kSums];
-    lbm::Counters c;
-    if ((rc = cuda_error(cudaMemcpyAsync(sums, res, sizeof(sums), cudaMemcpyDeviceToHost, h->stream), "diag copy")))
-        return rc;
-    if ((rc = cuda_error(cudaMemcpyAsync(&c, h->cnt, sizeof(c), cudaMemcpyDeviceToHost, h->stream), "diag copy")))
-        return rc;
-    if ((rc = sync_and_latch(h)) == LBM_ERR_CUDA || rc == LBM_ERR_TIMEOUT) return rc;
-    for (int q = 0; q < lbm::kSums; ++q) out[q] = sums[q];
-    out[5] = (double)c.clamps;
-    out[6] = (double)c.bad;
+    double got[8];
+    const int rc = lbm::diagnose(h, 0, h->nn, h->partials, got);
+    if (rc != LBM_OK && rc != LBM_ERR_NONPHYSICAL) return rc;
+    for (int q = 0; q < 7; ++q) out[q] = got[q];
     out[7] = (double)h->steps;
     return rc;
 }

@@ -65,9 +65,10 @@ int launch_sums(int nx, int ny, int nz, double rho_ref, double E_ref, const void
     kp.rho_ref = (R)rho_ref;
     kp.E_ref = (R)E_ref;
     // the caller's buffer holds set-major planes (the checkpoint layout)
+    const int blocks = lbm::reduce_blocks(kp.nn);
     lbm::reduce_kernel<Q, S, R, false>
-        <<<lbm::kReduceBlocks, lbm::kReduceThreads, 0, stream>>>((const S*)pop, kp, scratch);
-    lbm::reduce_final_kernel<<<1, 32, 0, stream>>>(scratch, lbm::kReduceBlocks, sums);
+        <<<blocks, lbm::kReduceThreads, 0, stream>>>((const S*)pop, kp.nn, 0, kp.nn, kp, scratch);
+    lbm::reduce_final_kernel<<<lbm::kSums, 32, 0, stream>>>(scratch, blocks, sums, nullptr);
     return lbm::cuda_error(cudaGetLastError(), "lbm_conservation_sums_noalloc launch");
 }
 

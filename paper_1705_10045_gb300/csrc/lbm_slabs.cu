@@ -42,7 +42,7 @@ struct lbm_slabs {
     std::vector<lbm_slab> plan;
     std::vector<lbm_handle*> h;
     double* tmp = nullptr;         // (D + 3) field planes of the largest slab
-    double* partials = nullptr;    // reduction partials, then kSums results
+    double* partials = nullptr;    // reduction partials, then 8 results
     long long steps = 0;
     cudaStream_t main = nullptr;   // the caller's stream, which every slab steps on
 };
@@ -211,76 +211,6 @@ int copy_crossing_rows(const void* src, void* dst, const RowTable& t, const Cros
     return cuda_error(cudaGetLastError(), "crossing copy launch");
 }
 
-
-// Conservation sums of nodes [i0, i0 + n) of a population buffer whose
-// arrays are nn apart: per-thread compensated sums in the arithmetic type,
-// combined in FP64 in a fixed order (as in the whole-domain reduction).
-template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(lbm::kReduceThreads) range_reduce_kernel(const S* __restrict__ pop, long long nn,
-                                                                          long long i0, long long n,
-                                                                          lbm::KParams<R> p,
-                                                                          double* __restrict__ partials) {
-    lbm::Kahan acc[lbm::kSums];   // FP64, compensated, as the whole-domain sums
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride) {
-        R rho, jx, jy, jz, E;
-        lbm::node_moments<Q, S, R>(pop, nn, i0 + t, p, rho, jx, jy, jz, E);
-        acc[0].add((double)rho);
-        acc[1].add((double)jx);
-        acc[2].add((double)jy);
-        acc[3].add((double)jz);
-        acc[4].add((double)E);
-    }
-    __shared__ double sh[lbm::kSums][lbm::kReduceThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < lbm::kSums; ++q) {
-        double v = lbm::warp_sum(acc[q].s - acc[q].c);
-        if (lane == 0) sh[q][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < lbm::kSums) {
-        lbm::Kahan b;
-        for (int w = 0; w < lbm::kReduceThreads / 32; ++w) b.add(sh[threadIdx.x][w]);
-        partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = b.s;
-    }
-}
-
-__global__ void __launch_bounds__(32) range_final_kernel(const double* __restrict__ partials, int nblocks,
-                                                         double* __restrict__ out) {
-    if (threadIdx.x < lbm::kSums) {
-        lbm::Kahan b;
-        for (int j = 0; j < nblocks; ++j) b.add(partials[(size_t)threadIdx.x * nblocks + j]);
-        out[threadIdx.x] = b.s;
-    }
-}
-
-template <int Q, typename S, typename R>
-int launch_range_sums(const lbm_handle* h, long long i0, long long n, double* partials, double* out) {
-    lbm::KParams<R> kp{};
-    kp.nn = h->nn;
-    kp.rho_ref = h->p.storage == LBM_STORE_FP16 ? (R)h->p.rho_ref : R(0);
-    kp.E_ref = h->p.storage == LBM_STORE_FP16 ? (R)h->p.E_ref : R(0);
-    range_reduce_kernel<Q, S, R><<<lbm::kReduceBlocks, lbm::kReduceThreads, 0, h->stream>>>(
-        (const S*)h->pop[h->cur], h->nn, i0, n, kp, partials);
-    range_final_kernel<<<1, 32, 0, h->stream>>>(partials, lbm::kReduceBlocks, out);
-    return cuda_error(cudaGetLastError(), "slab sums launch");
-}
-
-int range_sums(const lbm_handle* h, long long i0, long long n, double* partials, double* out) {
-    if (h->Q == 9) {
-        switch (h->p.storage) {
-            case LBM_STORE_FP64: return launch_range_sums<9, double, double>(h, i0, n, partials, out);
-            case LBM_STORE_FP32: return launch_range_sums<9, float, float>(h, i0, n, partials, out);
-            default: return launch_range_sums<9, __half, float>(h, i0, n, partials, out);
-        }
-    }
-    switch (h->p.storage) {
-        case LBM_STORE_FP64: return launch_range_sums<19, double, double>(h, i0, n, partials, out);
-        case LBM_STORE_FP32: return launch_range_sums<19, float, float>(h, i0, n, partials, out);
-        default: return launch_range_sums<19, __half, float>(h, i0, n, partials, out);
-    }
-}
 
 // global planes of slab s's local planes, in at most two runs (a periodic
 // domain wraps the first slab's lower halo to the top of the domain)
@@ -532,7 +462,7 @@ int lbm_slabs_create(const lbm_params* p, int count, lbm_slabs** out) {
                         "slab field allocation");
         if (!rc)
             rc = cuda_error(cudaMalloc((void**)&s->partials,
-                                       sizeof(double) * (size_t)(lbm::kSums * lbm::kReduceBlocks + lbm::kSums)),
+                                       sizeof(double) * (size_t)(lbm::kSums * lbm::kReduceBlocks + 8)),
                             "slab reduction scratch allocation");
     }
     if (rc) {
@@ -659,17 +589,10 @@ int lbm_slabs_diagnostics(lbm_slabs* s, double out[8]) {
     double tot[lbm::kSums] = {0}, comp[lbm::kSums] = {0};   // Kahan sums over the slabs
     double clamps = 0, bad = 0;
     int latched = LBM_OK;
-    double* res = s->partials + lbm::kSums * lbm::kReduceBlocks;
     for (int i = 0; i < s->count; ++i) {
         const lbm_slab& sl = s->plan[i];
-        lbm_handle* h = s->h[i];
-        int rc = range_sums(h, (long long)sl.lo * s->plane, (long long)sl.own * s->plane, s->partials, res);
-        double sums[lbm::kSums];
-        lbm::Counters c;
-        if (!rc) rc = cuda_error(cudaMemcpyAsync(sums, res, sizeof(sums), cudaMemcpyDeviceToHost, h->stream), "slab sums copy");
-        if (!rc) rc = cuda_error(cudaMemcpyAsync(&c, h->cnt, sizeof(c), cudaMemcpyDeviceToHost, h->stream), "slab counters copy");
-        if (rc) return rc;
-        rc = lbm_sync(h);   // waits for the copies; reports a latched device error
+        double sums[8];
+        const int rc = lbm::diagnose(s->h[i], (long long)sl.lo * s->plane, (long long)sl.own * s->plane, s->partials, sums);
         if (rc == LBM_ERR_NONPHYSICAL && !latched)
             latched = rc;
         else if (rc)
@@ -679,8 +602,8 @@ int lbm_slabs_diagnostics(lbm_slabs* s, double out[8]) {
             comp[q] = (t - tot[q]) - y;
             tot[q] = t;
         }
-        clamps += (double)c.clamps;
-        bad += (double)c.bad;
+        clamps += sums[5];
+        bad += sums[6];
     }
     for (int q = 0; q < lbm::kSums; ++q) out[q] = tot[q];
     out[5] = clamps;
