@@ -9,6 +9,7 @@
 #include "fused.cuh"
 #include "internal.h"
 #include "kernels.cuh"
+#include "phases.cuh"
 #include "strip.cuh"
 
 namespace lbm {
@@ -37,6 +38,8 @@ template <typename R> KParams<R> make_kparams(const lbm_handle* h) {
     k.step = (unsigned)h->steps;
     k.latent = (R)q.latent;
     k.coex = (const R*)h->coex;
+    k.inv_c_v = (R)(1.0 / q.c_v);
+    k.half_cv_chi = (R)(0.5 * q.c_v * q.chi);
     return k;
 }
 
@@ -91,7 +94,12 @@ template <typename R> struct BatchShape<19, R, 2> { static constexpr int TX = 32
 template <int Q, typename S, typename R> struct Impl {
     static constexpr int TX = FusedTile<Q, R>::TX, TY = FusedTile<Q, R>::TY, NP = FusedTile<Q, R>::NP;
     static constexpr bool SPLIT = FusedTile<Q, R>::SPLIT;
-    static int launches(const lbm_handle* h) { return h->p.step_kernel == LBM_STEP_THREE_LAUNCH ? 3 : 1; }
+    // FP64 steps in three phases (phases.cuh) where the handle has their planes
+    static constexpr bool kPhases = std::is_same<S, double>::value;
+    static bool phases(const lbm_handle* h) { return kPhases && h->ext && h->fault_drop <= 0; }
+    static int launches(const lbm_handle* h) {
+        return h->p.step_kernel == LBM_STEP_THREE_LAUNCH || phases(h) ? 3 : 1;
+    }
 
     // planes [m_lo, m_hi) collided; m_hi < 0: the handle's own range
     // (lbm_set_step_planes; all by default)
@@ -133,8 +141,44 @@ template <int Q, typename S, typename R> struct Impl {
         return s;
     }
 
+    // the step over the planes of G in three launches
+    static void launch_phase(lbm_handle* h, const KParams<R>& kp, const MarchGeom& G, const S* src, S* dst, int j) {
+        // the moments of two planes and the forces of one plane beyond the
+        // range, or of every plane
+        const int reach = 2 - j, len = G.m_hi - G.m_lo;
+        PhaseGeom g;
+        g.plane_n = G.na * G.nb;
+        g.nm = G.nm;
+        g.m_lo = G.m_lo;
+        g.m_hi = G.m_hi;
+        g.first = G.m_lo - reach;
+        g.count = len + 2 * reach;
+        if (h->p.wall) {
+            const int hi = std::min(g.first + g.count, G.nm);
+            g.first = std::max(g.first, 0);
+            g.count = hi - g.first;
+        } else if (g.count >= G.nm) {
+            g.first = 0;
+            g.count = G.nm;
+        } else if (g.first < 0) {
+            g.first += G.nm;
+        }
+        const unsigned grid = grid_for((long long)g.count * g.plane_n, 128);
+        R* fld = (R*)h->fld;
+        R* ext = (R*)h->ext;
+        if (j == 0) launch_after(phase_moments_kernel<Q, S, R>, grid, 128, 0, h->stream, src, fld, ext, kp, g, (Counters*)h->cnt);
+        if (j == 1) launch_after(phase_force_kernel<Q, S, R>, grid, 128, 0, h->stream, fld, ext, kp, g);
+        if (j == 2) launch_after(phase_collide_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, ext, kp, g);
+    }
+
     // the fused step over the planes of G, src -> dst (no buffer swap)
     static void launch_fused_range(lbm_handle* h, const KParams<R>& kp, const MarchGeom& G, const S* src, S* dst) {
+        if constexpr (kPhases) {
+            if (phases(h)) {
+                for (int j = 0; j < 3; ++j) launch_phase(h, kp, G, src, dst, j);
+                return;
+            }
+        }
         if constexpr (kStrips) {
             if (h->fault_drop <= 0) {
                 const StripGeom g = strip_geometry(G);
@@ -181,6 +225,13 @@ template <int Q, typename S, typename R> struct Impl {
     // launch j of one time step; the last launch of a step swaps the buffers
     static void launch(lbm_handle* h, const KParams<R>& kp, int j) {
         if (h->p.step_kernel != LBM_STEP_THREE_LAUNCH) {
+            if constexpr (kPhases) {
+                if (phases(h)) {
+                    launch_phase(h, kp, geometry(h), (const S*)h->pop[h->cur], (S*)h->pop[h->cur ^ 1], j);
+                    if (j == 2) h->cur ^= 1;
+                    return;
+                }
+            }
             launch_fused(h, kp);
             return;
         }
@@ -417,12 +468,12 @@ template <int Q> int Backend<Q>::profile(lbm_handle* h, int n, double* ms, int c
 template <int Q> const char* Backend<Q>::launch_name(const lbm_handle* h, int j) {
     static const char* three[] = {"fields_kernel", "force_kernel", "collide_kernel"};
     if (h->p.step_kernel == LBM_STEP_THREE_LAUNCH) return j >= 0 && j < 3 ? three[j] : "";
+    static const char* phase[] = {"phase_moments_kernel", "phase_force_kernel", "phase_collide_kernel"};
+    if (launches(h) == 3) return j >= 0 && j < 3 ? phase[j] : "";
     if (j != 0) return "";
     return Q == 9 && h->p.storage != LBM_STORE_FP64 ? "strip_step_kernel" : "fused_step_kernel";
 }
-template <int Q> int Backend<Q>::launches(const lbm_handle* h) {
-    return h->p.step_kernel == LBM_STEP_THREE_LAUNCH ? 3 : 1;
-}
+template <int Q> int Backend<Q>::launches(const lbm_handle* h) { LBM_DISPATCH(h, launches(h)); }
 template <int Q> int Backend<Q>::init(lbm_handle* h, const double* rho, const double* u, const double* eps) {
     LBM_DISPATCH(h, init(h, rho, u, eps));
 }
@@ -455,6 +506,9 @@ template <int Q> size_t Backend<Q>::desc_bytes(int storage) {
 
 template <int Q> size_t Backend<Q>::field_bytes(int storage) {
     return (size_t)F_COUNT * (storage == LBM_STORE_FP64 ? sizeof(double) : sizeof(float));
+}
+template <int Q> size_t Backend<Q>::phase_bytes(int storage) {
+    return storage == LBM_STORE_FP64 ? (size_t)X_COUNT * sizeof(double) : 0;
 }
 
 #undef LBM_DISPATCH

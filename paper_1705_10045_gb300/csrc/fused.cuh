@@ -29,10 +29,16 @@
 // TX x 1.
 //
 // Index arithmetic is kept out of the inner loops: the wrapped ring
-// coordinates of a CTA are tabulated once in shared memory, and each
-// consumer thread precomputes the +-1 node offsets of its node along every
-// axis.  The force stencil and the collision work on opposite-direction pairs
-// (c_{k+1} = -c_k), which share the even part of every term.
+// coordinates of a CTA are tabulated once in shared memory, buffer slots come
+// from one remainder per plane, pair pointers walk from one direction's array
+// to the next, and each consumer thread precomputes the +-1 node offsets of
+// its node along every axis.  The force stencil and the collision (node.cuh)
+// work on opposite-direction pairs (c_{k+1} = -c_k), which share the even part
+// of every term, and the collision on both sets at once (f32x2).  384 x 384 x
+// 256 D3Q19, a remainder per buffer access and scalar arithmetic -> this: FP32
+// 2628 -> 2545 us (43.3 -> 38.7 warp instructions per node), FP16 storage
+// 2175 -> 2014 (46.5 -> 42.1).  Carrying the slots from plane to plane instead
+// spilled (80 registers): 2728 / 2152.
 #pragma once
 
 #include "node.cuh"
@@ -138,8 +144,6 @@ __device__ __forceinline__ int wrapi(int i, int n) {
     return i < 0 ? i + n : i;
 }
 
-__device__ __forceinline__ int slotn(int m, int n) { return ((m % n) + n) % n; }
-
 // Coordinate of a ring row or column: wrapped on a periodic axis, the mirror
 // node across a wall (clamped into the axis for ring nodes of a ragged tile
 // that lie further out; their values are never used).
@@ -165,6 +169,7 @@ __device__ __forceinline__ int wall_edges(const KParams<R>& p, int Q, int ga, in
 template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool SPLIT = false> struct FusedStages {
     using V = Vel<Q>;
     using M = MVel<Q>;
+    using Math = NodeMath<Q, S, R>;
     using Sh = FusedShape<TX, TY, SPLIT>;
     static constexpr int RB = Sh::RB, RW = Sh::RW, RH = Sh::RH, R_ = Sh::R, FW = Sh::FW, FB = Sh::FB, F_ = Sh::F;
 
@@ -181,381 +186,174 @@ template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool 
     int plane_n;
     unsigned step;   // step counter of this launch (seeds FP16 stochastic rounding)
 
-    // the pair (N_k, g_k) at pair index i of q.  With shifted storage (FP16)
-    // the stages work on the stored values N_k - w_k rho_ref, g_k - w_k E_ref
-    // themselves: the moments add rho_ref and E_ref once, and the collision
-    // writes shifted values (see c_stage), so no value is shifted on its own.
-    static constexpr bool kSh = Store<S, R>::kShifted;
-    __device__ static void ld2(const S* q, size_t i, R sN, R sG, R& a, R& b) {
-        if constexpr (kSh) {
-            if (COH) Store<S, R>::load2_coh_raw(q, i, a, b);
-            else Store<S, R>::load2_raw(q, i, a, b);
-        } else {
-            if (COH) Store<S, R>::load2_coh(q, i, sN, sG, a, b);
-            else Store<S, R>::load2(q, i, sN, sG, a, b);
-        }
-    }
-    __device__ static void ld2_last(const S* q, size_t i, R sN, R sG, R& a, R& b) {
-        if constexpr (kSh) {
-            if (COH) Store<S, R>::load2_last_coh_raw(q, i, a, b);
-            else Store<S, R>::load2_last_raw(q, i, a, b);
-        } else {
-            if (COH) Store<S, R>::load2_last_coh(q, i, sN, sG, a, b);
-            else Store<S, R>::load2_last(q, i, sN, sG, a, b);
-        }
-    }
     __device__ R& phi(int slot, int r) const { return phis[slot * R_ + r]; }
     __device__ R& rut(int slot, int f, int r) const { return ruts[(slot * Sh::kRut + f) * F_ + r]; }
     __device__ R& du(int slot, int c, int r) const { return dus[(slot * 3 + c) * F_ + r]; }
     // Buffer slots are keyed by the unwrapped plane index the M stage loaded
-    // (a periodic plane -1 holds the data of plane nm-1); across a wall a
-    // stencil read goes to the mirror plane instead.
-    __device__ int mplane(int m) const {
-        if (!p->wall) return m;
-        return m < 0 ? -1 - m : (m >= G.nm ? 2 * G.nm - 1 - m : m);
-    }
+    // (a periodic plane -1 holds the data of plane nm-1): one remainder per
+    // plane, the neighbouring planes' slots from it (a remainder per access
+    // would cost a dozen instructions each).
+    struct Slots {
+        int m, phi, rut;   // plane, its Phi slot and its rho/u/T slot
+        __device__ explicit Slots(int plane) : m(plane) {   // plane >= -3
+            const unsigned u = (unsigned)(plane + 3 * Sh::kPhiSlots * Sh::kRutSlots);
+            phi = (int)(u % Sh::kPhiSlots);
+            rut = (int)(u % Sh::kRutSlots);
+        }
+        static_assert(Sh::kDuSlots == 4, "du slots by mask");
+        __device__ int du(int d = 0) const { return (m + d) & 3; }
+        __device__ int phi_at(int d) const {   // |d| < kPhiSlots
+            const int s = phi + d;
+            return s < 0 ? s + Sh::kPhiSlots : (s >= Sh::kPhiSlots ? s - Sh::kPhiSlots : s);
+        }
+        __device__ int rut_at(int d) const {   // |d| < kRutSlots
+            const int s = rut + d;
+            return s < 0 ? s + Sh::kRutSlots : (s >= Sh::kRutSlots ? s - Sh::kRutSlots : s);
+        }
+    };
 
-    // M: moments of plane m on the ring region, ring nodes t, t + nt, ...
-    __device__ void m_stage(int m, int t, int nt) const {
-        const int plane_off = wrapi(m, G.nm) * plane_n;
-        const int sp = slotn(m, Sh::kPhiSlots), sr = slotn(m, Sh::kRutSlots);
-        for (int r = t; r < R_; r += nt) m_node(plane_off, sp, sr, r);
+    // M: moments of plane sl.m on the ring region, ring nodes t, t + nt, ...
+    __device__ void m_stage(const Slots& sl, int plane_off, int t, int nt) const {
+        for (int r = t; r < R_; r += nt) m_ring(sl.phi, sl.rut, plane_off, r);
     }
     // the same for the border nodes only (SPLIT: the consumers take the tile)
-    __device__ void m_border(int m, int t, int nt) const {
-        const int plane_off = wrapi(m, G.nm) * plane_n;
-        const int sp = slotn(m, Sh::kPhiSlots), sr = slotn(m, Sh::kRutSlots);
-        for (int q = t; q < Sh::kBorder; q += nt) m_node(plane_off, sp, sr, Sh::border_ring(q));
+    __device__ void m_border(const Slots& sl, int plane_off, int t, int nt) const {
+        for (int q = t; q < Sh::kBorder; q += nt) m_ring(sl.phi, sl.rut, plane_off, Sh::border_ring(q));
     }
-    // the moments of tile node (ta, tb) of plane m
-    __device__ void m_interior(int m, int ta, int tb) const {
-        m_node<true>(wrapi(m, G.nm) * plane_n, slotn(m, Sh::kPhiSlots), slotn(m, Sh::kRutSlots),
-                     (tb + RB) * RW + ta + 2);
+    __device__ __forceinline__ void m_ring(int sp, int sr, int plane_off, int r) const {
+        const int ra = r % RW, rb = r / RW, fa = ra - 1, fb = rb - (RB - FB);
+        const bool inner = fa >= 0 && fa < FW && fb >= 0 && fb < Sh::FH;
+        m_node<kUse>(plane_off + ring_b[rb] + ring_a[ra], sp, sr, r, inner ? fb * FW + fa : -1);
     }
-    // Phi of ring node r, and rho, u, T if r lies in the 1-ring region.
-    // KEEP: the node is the caller's own, reloaded by its C stage three
-    // planes later, so its lines get the L2 evict-last hint.
-    template <bool KEEP = false>
-    __device__ __forceinline__ void m_node(int plane_off, int sp, int sr, int r) const {
-        {
-            const int ra = r % RW, rb = r / RW;
-            const size_t n = (size_t)(plane_off + ring_b[rb] + ring_a[ra]);
-            if constexpr (kSh) {
-                // shifted FP16 storage: the sums take the halves of the pair
-                // words directly (the same values as widening them first)
-                using H = Store<S, R>;
-                unsigned w[Q];
+    // Moments of node n: Phi at ring index r, and rho, u, T at 1-ring index f
+    // (f < 0: the node lies outside the 1-ring region).
+    template <LoadUse U> __device__ __forceinline__ void m_node(int n, int sp, int sr, int r, int f) const {
+        Pop<S> w[Q];
 #pragma unroll
-                for (int k = 0; k < Q; ++k)
-                    w[k] = COH ? H::word_coh(src, pair_index(k, nn, n)) : H::word(src, pair_index(k, nn, n));
-                R rho = H::lo(w[0]), ja = R(0), jb = R(0), jm = R(0), E = H::hi(w[0]);
-                bool new_a = true, new_b = true, new_m = true;
-#pragma unroll
-                for (int k = 1; k < Q; k += 2) {
-                    const R x = H::lo(w[k]);
-                    const R s = H::add_lo(w[k + 1], x), dn = H::sub_lo(w[k + 1], x);   // x + y and y - x
-                    rho += s;
-                    if (M::a(k) != 0) { const R t = M::a(k) > 0 ? -dn : dn; ja = new_a ? t : ja + t; new_a = false; }
-                    if (M::b(k) != 0) { const R t = M::b(k) > 0 ? -dn : dn; jb = new_b ? t : jb + t; new_b = false; }
-                    if (M::m(k) != 0) { const R t = M::m(k) > 0 ? -dn : dn; jm = new_m ? t : jm + t; new_m = false; }
-                }
-#pragma unroll
-                for (int k = 1; k < Q; ++k) E = H::add_hi(w[k], E);
-                // sums of shifted values: sum_k w_k = 1, sum_k w_k c_k = 0
-                rho += p->rho_ref;
-                E += p->E_ref;
-                m_finish(sp, sr, r, rho, ja, jb, jm, E);
-                return;
-            } else {
-                R fN[Q], fG[Q];
-#pragma unroll
-                for (int k = 0; k < Q; ++k)
-                    if (KEEP && !COH)
-                        Store<S, R>::load2_keep(src, pair_index(k, nn, n), R(V::w(k)) * p->rho_ref,
-                                                R(V::w(k)) * p->E_ref, fN[k], fG[k]);
-                    else
-                        ld2(src, pair_index(k, nn, n), R(V::w(k)) * p->rho_ref, R(V::w(k)) * p->E_ref, fN[k], fG[k]);
-                // opposite directions k, k+1 pair up: their sum enters rho, their
-                // difference the momentum along c_k (each sum starts at its
-                // first term)
-                R rho = fN[0], ja = R(0), jb = R(0), jm = R(0), E = fG[0];
-                bool new_a = true, new_b = true, new_m = true;
-#pragma unroll
-                for (int k = 1; k < Q; k += 2) {
-                    const R s = fN[k] + fN[k + 1], d = fN[k] - fN[k + 1];
-                    rho += s;
-                    if (M::a(k) != 0) { const R t = M::a(k) > 0 ? d : -d; ja = new_a ? t : ja + t; new_a = false; }
-                    if (M::b(k) != 0) { const R t = M::b(k) > 0 ? d : -d; jb = new_b ? t : jb + t; new_b = false; }
-                    if (M::m(k) != 0) { const R t = M::m(k) > 0 ? d : -d; jm = new_m ? t : jm + t; new_m = false; }
-                }
-#pragma unroll
-                for (int k = 1; k < Q; ++k) E += fG[k];
-                m_finish(sp, sr, r, rho, ja, jb, jm, E);
-            }
-        }
-    }
-    // Phi of ring node r from its moments, and rho, u, T if r lies in the
-    // 1-ring region
-    __device__ __forceinline__ void m_finish(int sp, int sr, int r, R rho, R ja, R jb, R jm, R E) const {
-        const R third = R(1.0 / 3.0);
-        const int ra = r % RW, rb = r / RW;
-        const R T = E / (rho * p->c_v);
-        const R U = fma(-rho, third, eos_pressure(*p, rho, T));
-        phi(sp, r) = U < R(0) ? sqrt(-U) : R(0);
-        const int fa = ra - 1, fb = rb - (RB - FB);
-        if (fa >= 0 && fa < FW && fb >= 0 && fb < Sh::FH) {
-            const int f = fb * FW + fa;
-            const R inv_rho = R(1) / rho;
-            rut(sr, 0, f) = rho;
-            rut(sr, 1, f) = ja * inv_rho;
-            rut(sr, 2, f) = jb * inv_rho;
-            rut(sr, 3, f) = jm * inv_rho;
+        for (int k = 0; k < Q; ++k) w[k] = load_pop<COH, U>(src + 2 * ((size_t)k * nn), (size_t)(unsigned)n);
+        const Moments<R> o = Math::moments(w, *p);
+        const R inv = Math::kF64 || f >= 0 ? R(1) / o.rho : R(0);
+        const R T = Math::temperature(*p, o.rho, inv, o.E);
+        phi(sp, r) = Math::phi_of(Math::potential(o.rho, Math::pressure(*p, o.rho, T)));
+        if (f >= 0) {
+            rut(sr, 0, f) = o.rho;
+            rut(sr, 1, f) = o.ja * inv;
+            rut(sr, 2, f) = o.jb * inv;
+            rut(sr, 3, f) = o.jm * inv;
             rut(sr, 4, f) = T;
         }
     }
 
-    // F: du = F/rho on the 1-ring region of plane f, region nodes t, t + nt, ...
-    __device__ void f_stage(int f, int t, int nt) const {
-        const int sp0 = slotn(f, Sh::kPhiSlots), spm = slotn(mplane(f - 1), Sh::kPhiSlots),
-                  spp = slotn(mplane(f + 1), Sh::kPhiSlots);
-        const int sr = slotn(f, Sh::kRutSlots), sd = slotn(f, Sh::kDuSlots);
-        const R A = p->A, B = R(1) - R(2) * p->A, inv_alpha = R(1.0 / V::alpha);
-        const R gv[3] = {p->g[0], Q == 9 ? R(0) : p->g[1], Q == 9 ? p->g[1] : p->g[2]};
-        const R G2 = R(V::G(Q - 1));   // next-nearest weight (1/4 or 1/2)
+    // F: du = F/rho on the 1-ring region of plane sl.m, region nodes t, t + nt, ...
+    // Across a wall the stencil reads the mirror plane, the plane itself.
+    __device__ void f_stage(const Slots& sl, int t, int nt) const {
+        const int sp0 = sl.phi, spm = p->wall && sl.m == 0 ? sp0 : sl.phi_at(-1),
+                  spp = p->wall && sl.m == G.nm - 1 ? sp0 : sl.phi_at(1);
+        const int sd = sl.du();
         for (int r = t; r < F_; r += nt) {
-            const int ra = r % FW + 1, rb = r / FW + (RB - FB);
-            // opposite directions pair up: G Phi(x+e) e + G Phi(x-e)(-e) = G (Phi+ - Phi-) e,
-            // and the Phi^2 term is G (Phi+ - Phi-)(Phi+ + Phi-) e
-            R n1[3] = {0, 0, 0}, n2[3] = {0, 0, 0}, q1[3] = {0, 0, 0}, q2[3] = {0, 0, 0};
-#pragma unroll
-            for (int k = 1; k < Q; k += 2) {
-                const int s_p = M::m(k) == 0 ? sp0 : (M::m(k) > 0 ? spp : spm);
-                const int s_m = M::m(k) == 0 ? sp0 : (M::m(k) > 0 ? spm : spp);
-                const R pp = phi(s_p, (rb + M::b(k)) * RW + ra + M::a(k));
-                const R pm = phi(s_m, (rb - M::b(k)) * RW + ra - M::a(k));
-                const R d = pp - pm, sum = pp + pm;
-                const bool nearest = M::a(k) * M::a(k) + M::b(k) * M::b(k) + M::m(k) * M::m(k) == 1;
-                R* s1 = nearest ? n1 : q1;
-                R* s2 = nearest ? n2 : q2;
-                // s1 += +-d (Phi+ + Phi-) as one fused multiply-add per axis
-                if (M::a(k) == 1) { s1[0] = fma(d, sum, s1[0]); s2[0] += d; }
-                else if (M::a(k) == -1) { s1[0] = fma(-d, sum, s1[0]); s2[0] -= d; }
-                if (M::b(k) == 1) { s1[1] = fma(d, sum, s1[1]); s2[1] += d; }
-                else if (M::b(k) == -1) { s1[1] = fma(-d, sum, s1[1]); s2[1] -= d; }
-                if (M::m(k) == 1) { s1[2] = fma(d, sum, s1[2]); s2[2] += d; }
-                else if (M::m(k) == -1) { s1[2] = fma(-d, sum, s1[2]); s2[2] -= d; }
-            }
-            const R rho = rut(sr, 0, r), ph0 = phi(sp0, rb * RW + ra);
-            const R scale = inv_alpha / rho, Bph0 = B * ph0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const R s1 = fma(G2, q1[a], n1[a]), s2 = fma(G2, q2[a], n2[a]);
-                du(sd, a, r) = fma(fma(A, s1, Bph0 * s2), scale, gv[a]);
-            }
+            const int at = (r / FW + (RB - FB)) * RW + r % FW + 1;
+            const R rho = rut(sl.rut, 0, r);
+            R d[3];
+            Math::force(*p, [&](int a, int b, int m) {
+                return phi(m == 0 ? sp0 : (m > 0 ? spp : spm), at + b * RW + a);
+            }, rho, Math::kF64 ? R(1) / rho : R(0), d);
+            du(sd, 0, r) = d[0];
+            du(sd, 1, r) = d[1];
+            du(sd, 2, r) = d[2];
         }
     }
 
-    // C: energy change, collision and push of the node (ta, tb) of plane c.
+    // C: energy change, collision and push of the node at 1-ring index fc and
+    // index n_ab of its plane, plane sl.m.
     // edge: walls next to the node across the tile plane (bit 0 / 1: the low /
     // high wall of axis a, bit 2 / 3: of axis b), from wall_edges().
     // XW: the domain may have walls on the tile-plane axes (false: edge is 0
     // and the wall handling across the tile compiles away).
     template <bool XW>
-    __device__ void c_stage(int c, int ta, int tb, int n_ab, int dA_m, int dA_p, int dB_m, int dB_p, int edge_in,
-                            Counters* cnt) const {
-        const int edge = XW ? edge_in : 0;
-        const bool walls = p->wall;
+    __device__ void c_stage(const Slots& sl, int fc, int n_ab, int dA_m, int dA_p, int dB_m, int dB_p,
+                            int edge_in, Counters* cnt) const {
+        const int edge = XW ? edge_in : 0, c = sl.m;
         const int nm = G.nm;
-        const R third = R(1.0 / 3.0);
+        const bool gu = p->wall && c == nm - 1, gd = p->wall && c == 0;
         // the node's populations first: their loads are in flight while the
         // finite differences below read shared memory.  The reload is the last
         // use of these lines on this SM, so it does not allocate them in L1.
-        // The pointer walks from one direction's pair array to the next.
-        // With shifted FP16 storage the reload stays packed (one 32-bit word
-        // per pair, half the registers) and each half is widened where it is
-        // used.
+        // With FP16 storage it stays packed (one 32-bit word per pair) and
+        // each half is widened where it is used.
         const int n = c * plane_n + n_ab;
-        R fv[Q], hv[Q];
-        unsigned wv[Q];
-        {
-            const S* q = src + 2 * (size_t)n;
+        Pop<S> w[Q];
 #pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                if constexpr (kSh) wv[k] = COH ? Store<S, R>::word_last_coh(q, 0) : Store<S, R>::word_last(q, 0);
-                else ld2_last(q, 0, R(V::w(k)) * p->rho_ref, R(V::w(k)) * p->E_ref, fv[k], hv[k]);
-                q += 2 * nn;
-            }
-        }
-        auto fvk = [&](int k) -> R {   // N_k (stored, shifted value with FP16)
-            if constexpr (kSh) return __half2float(__ushort_as_half((unsigned short)(wv[k] & 0xFFFFu)));
-            else return fv[k];
-        };
-        auto hvk = [&](int k) -> R {   // g_k
-            if constexpr (kSh) return __half2float(__ushort_as_half((unsigned short)(wv[k] >> 16)));
-            else return hv[k];
-        };
-        const int sr = slotn(c, Sh::kRutSlots), sd = slotn(c, Sh::kDuSlots);
-        const int fc = (tb + FB) * FW + ta + 1;        // 1-ring index of the node
+        { const S* q = src + 2 * (size_t)n;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) { w[k] = load_pop<COH, kUseLast>(q, 0); q += 2 * nn; } }
+        const int sr = sl.rut, sd = sl.du();
         const R rho = rut(sr, 0, fc), T = rut(sr, 4, fc);
         const R u[3] = {rut(sr, 1, fc), rut(sr, 2, fc), rut(sr, 3, fc)};
         const R dv[3] = {du(sd, 0, fc), du(sd, 1, fc), du(sd, 2, fc)};
 
-        // finite-difference dE along a, b and the march axis (Sec. 4, Sec. 6.2)
-        R div = 0, cond = 0;
-        const R lc = conductivity(*p, rho), half_lc = lc * R(0.5);
-        // one axis of the differences; g: bit 0 / 1 the low / high neighbour is
-        // the ghost beyond a wall, whose values are then own_u (normal
-        // velocity), T_lo / T_hi and the node's own density
-        auto axis = [&](R uu, R ud, R Tu, R Td, R ru, R rd, int g = 0, R own_u = R(0), R T_lo = R(0),
-                        R T_hi = R(0)) {
+        // finite-difference neighbours along a, b and the march axis: ring
+        // nodes, or (only for nodes beside a wall) the node itself mirrored
+        // across it: normal velocity negated, T mirrored or reflected about
+        // the wall temperature
+        constexpr int N = V::D;
+        typename Math::Axis ax[N];
+        auto across = [&](int j, int a, int step, int g, const int* fixed, const R* Tw) {
+            ax[j] = {::fma(du(sd, a, fc + step), R(0.5), rut(sr, 1 + a, fc + step)),
+                     ::fma(du(sd, a, fc - step), R(0.5), rut(sr, 1 + a, fc - step)), rut(sr, 4, fc + step),
+                     rut(sr, 4, fc - step), rut(sr, 0, fc + step), rut(sr, 0, fc - step)};
             if (g) {
-                if (g & 2) { uu = own_u; Tu = T_hi; ru = rho; }
-                if (g & 1) { ud = own_u; Td = T_lo; rd = rho; }
+                const R own = -::fma(dv[a], R(0.5), u[a]);
+                if (g & 2) { ax[j].uu = own; ax[j].Tu = fixed[1] ? R(2) * Tw[1] - T : T; ax[j].ru = rho; }
+                if (g & 1) { ax[j].ud = own; ax[j].Td = fixed[0] ? R(2) * Tw[0] - T : T; ax[j].rd = rho; }
             }
-            div = fma(uu - ud, R(0.5), div);
-            // face conductivities, the mean of the two nodes'
-            const R lu = fma(conductivity(*p, ru), R(0.5), half_lc);
-            const R ld = fma(conductivity(*p, rd), R(0.5), half_lc);
-            cond = fma(-ld, T - Td, fma(lu, Tu - T, cond));
         };
-        // axes across the tile: neighbouring ring nodes, or (only for nodes
-        // beside a wall) the node itself mirrored across it: normal velocity
-        // negated, T mirrored or reflected about the wall temperature
-        axis(fma(du(sd, 0, fc + 1), R(0.5), rut(sr, 1, fc + 1)), fma(du(sd, 0, fc - 1), R(0.5), rut(sr, 1, fc - 1)),
-             rut(sr, 4, fc + 1), rut(sr, 4, fc - 1), rut(sr, 0, fc + 1), rut(sr, 0, fc - 1), edge & 3,
-             -fma(dv[0], R(0.5), u[0]), p->T_fixed_x[0] ? R(2) * p->T_x[0] - T : T,
-             p->T_fixed_x[1] ? R(2) * p->T_x[1] - T : T);
-        if (Q == 19)
-            axis(fma(du(sd, 1, fc + FW), R(0.5), rut(sr, 2, fc + FW)), fma(du(sd, 1, fc - FW), R(0.5), rut(sr, 2, fc - FW)),
-                 rut(sr, 4, fc + FW), rut(sr, 4, fc - FW), rut(sr, 0, fc + FW), rut(sr, 0, fc - FW), (edge >> 2) & 3,
-                 -fma(dv[1], R(0.5), u[1]), p->T_fixed_y[0] ? R(2) * p->T_y[0] - T : T,
-                 p->T_fixed_y[1] ? R(2) * p->T_y[1] - T : T);
-        {   // march axis: neighbouring planes, or the node itself mirrored across a wall
-            const bool gu = walls && c + 1 >= nm, gd = walls && c - 1 < 0;
-            const int su = slotn(c + 1, Sh::kRutSlots), sdn = slotn(c - 1, Sh::kRutSlots);
-            const int du_u = slotn(c + 1, Sh::kDuSlots), du_d = slotn(c - 1, Sh::kDuSlots);
-            const R own = -fma(dv[2], R(0.5), u[2]);
-            const R uu = gu ? own : fma(du(du_u, 2, fc), R(0.5), rut(su, 3, fc));
-            const R ud = gd ? own : fma(du(du_d, 2, fc), R(0.5), rut(sdn, 3, fc));
-            const R Tu = gu ? (p->T_fixed_hi ? R(2) * p->T_hi - T : T) : rut(su, 4, fc);
-            const R Td = gd ? (p->T_fixed_lo ? R(2) * p->T_lo - T : T) : rut(sdn, 4, fc);
-            const R ru = gu ? rho : rut(su, 0, fc);
-            const R rd = gd ? rho : rut(sdn, 0, fc);
-            axis(uu, ud, Tu, Td, ru, rd);
+        across(0, 0, 1, edge & 3, p->T_fixed_x, p->T_x);
+        if (Q == 19) across(1, 1, FW, (edge >> 2) & 3, p->T_fixed_y, p->T_y);
+        {
+            const int su = sl.rut_at(1), sdn = sl.rut_at(-1), du_u = sl.du(1), du_d = sl.du(-1);
+            const R own = -::fma(dv[2], R(0.5), u[2]);
+            ax[N - 1].uu = gu ? own : ::fma(du(du_u, 2, fc), R(0.5), rut(su, 3, fc));
+            ax[N - 1].ud = gd ? own : ::fma(du(du_d, 2, fc), R(0.5), rut(sdn, 3, fc));
+            ax[N - 1].Tu = gu ? (p->T_fixed_hi ? R(2) * p->T_hi - T : T) : rut(su, 4, fc);
+            ax[N - 1].Td = gd ? (p->T_fixed_lo ? R(2) * p->T_lo - T : T) : rut(sdn, 4, fc);
+            ax[N - 1].ru = gu ? rho : rut(su, 0, fc);
+            ax[N - 1].rd = gd ? rho : rut(sdn, 0, fc);
         }
-        const R P = eos_pressure(*p, rho, T);
-        R dE = 0;
-        if (p->pressure_work) dE += -P * div;
-        if (p->conduction) dE += cond;
-        if (p->latent != R(0)) dE += latent_heat(*p, rho, T, div);
-        if (fma(-rho, third, P) >= R(0)) atomicAdd(&cnt->clamps, 1ull);
+        const R P = Math::pressure(*p, rho, T);
+        const R dE = Math::energy_change(*p, rho, T, P, ax, N);
+        const R E = Math::energy(w, *p);
+        const bool clamp = Math::potential(rho, P) >= R(0), bad = !(Math::positive(rho) && Math::positive(E));
+        if (clamp || bad) {
+            if (clamp) atomicAdd(&cnt->clamps, 1ull);
+            if (bad) atomicAdd(&cnt->bad, 1ull);
+        }
 
-        R E = hvk(0);
-        if constexpr (kSh) {
-#pragma unroll
-            for (int k = 1; k < Q; ++k) E = Store<S, R>::add_hi(wv[k], E);
-            E += p->E_ref;
-        } else {
-#pragma unroll
-            for (int k = 1; k < Q; ++k) E += hvk(k);
-        }
-        if (!(finite_pos(rho) && finite_pos(E))) atomicAdd(&cnt->bad, 1ull);
-        const R dEoverE = dE / E;
         // node offsets of x + c_k: +-1 along a and b (periodic), along the
         // march axis periodic or bounced at a wall
         const int dM_m = (c == 0 ? nm - 1 : -1) * plane_n, dM_p = (c == nm - 1 ? 1 - nm : 1) * plane_n;
-        const bool wall_lo = walls && c == 0, wall_hi = walls && c == nm - 1;
-        const bool edge_a_lo = edge & 1, edge_a_hi = edge & 2, edge_b_lo = edge & 4, edge_b_hi = edge & 8;
-
-        // Collision, Eq. (lbe)/(edm)/(gk), written per node as
-        //   N*_k = (1 - omega) N_k + rho (omega e0_k + de_k)
-        //   g*_k = (1 - omega_E + dE/E) g_k + E (omega_E e0_k + [pseudoforce] de_k)
-        // with e0 = N^eq(rho,u)/rho and de = (N^eq(rho,u+du) - N^eq(rho,u))/rho.
-        // With v = u + du, s = c_k.u and t = c_k.v, Eq. (feq) gives
-        //   e0_k = w_k (b0 + 4.5 s^2 + 3 s),   de_k = w_k (db + 4.5 (t^2 - s^2) + 3 (t - s))
-        // (b0 = 1 - 1.5 u.u, db = -1.5 (v.v - u.u) = -1.5 du.(2u + du)), so
-        //   rho (omega e0_k + de_k) = w_k K + 4.5 w_k [P s^2 + rho t^2] + 3 w_k [P s + rho t]
-        // with K = rho omega b0 + rho db and P = rho omega - rho; the same holds
-        // for g with (E omega_E, E_pf) in place of (rho omega, rho).  Opposite
-        // directions k, k+1 (c -> -c) share the even part and flip the odd one.
-        // The factors w K, 4.5 w P, ... are formed once for the nearest
-        // directions and scaled by w2/w1 (1/2 on D3Q19, 1/4 on D2Q9: exact) for
-        // the next-nearest.  Products that feed a sum are written as explicit
-        // fused multiply-adds, so every kernel that runs this code rounds them
-        // the same way.
-        const R usq = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
-        const R dsq = fma(dv[0], fma(R(2), u[0], dv[0]), fma(dv[1], fma(R(2), u[1], dv[1]), dv[2] * fma(R(2), u[2], dv[2])));
-        const R base0 = fma(R(-1.5), usq, R(1)), dbase = R(-1.5) * dsq;
-        const R om = p->omega, omE = p->omega_E;
-        const R fN = R(1) - om, fG = R(1) - omE + dEoverE;
-        const R rho_om = rho * om, E_omE = E * omE, E_pf = p->pseudoforce ? E : R(0);
-        // shifted storage: with N_k = N'_k + w_k rho_ref and g_k = g'_k + w_k E_ref
-        //   N*'_k = (1 - omega) N'_k + rho (omega e0_k + de_k) - omega w_k rho_ref
-        //   g*'_k = fG g'_k + E (omega_E e0_k + [pf] de_k) + (fG - 1) w_k E_ref
-        // so the shifts enter K as nsh and gsh
-        const R nsh = kSh ? -om * p->rho_ref : R(0), gsh = kSh ? (fG - R(1)) * p->E_ref : R(0);
-        const R KN = kSh ? fma(rho_om, base0, fma(rho, dbase, nsh)) : fma(rho_om, base0, rho * dbase);
-        const R KG = kSh ? fma(E_omE, base0, fma(E_pf, dbase, gsh)) : fma(E_omE, base0, E_pf * dbase);
-        const R PN = rho_om - rho, PG = E_omE - E_pf;
-        const R v[3] = {u[0] + dv[0], u[1] + dv[1], u[2] + dv[2]};
         const unsigned nbits = Store<S, R>::kStochastic ? node_bits(step, (unsigned)n) : 0u;
-        S* dk = dst + 2 * (size_t)n;        // pair k of the node's slot (walks over k)
+        Pop<S>* out = reinterpret_cast<Pop<S>*>(dst);
+        Pop<S>* dk = out + n;
         // the collision and push, instantiated once for planes next to a wall
         // (WALL: some directions bounce back) and once for all other planes
         auto collide = [&](auto wall_tag) {
             constexpr bool WALL = decltype(wall_tag)::value;
-            // a: rho (omega e0 + de), b: E (omega_E e0 + [pseudoforce] de) of direction k
-            auto emit = [&](int k, R a, R b, R fv, R hvk) {
-                const R fo = fma(fv, fN, a);
-                const R ho = fma(hvk, fG, b);
-                // push to x + c_k, or bounce back at a wall on the march axis
-                const bool bounce = WALL && ((M::m(k) == -1 && wall_lo) || (M::m(k) == 1 && wall_hi) ||
-                                             (M::a(k) == -1 && edge_a_lo) || (M::a(k) == 1 && edge_a_hi) ||
-                                             (M::b(k) == -1 && edge_b_lo) || (M::b(k) == 1 && edge_b_hi));
+            Math::collide(*p, rho, E, u, dv, dE, [&](int k) { return w[k]; }, [&](int k, Two<R> v) {
+                // push to x + c_k, or bounce back at a wall
+                const bool bounce = WALL && ((M::m(k) == -1 && gd) || (M::m(k) == 1 && gu) ||
+                                             (M::a(k) == -1 && (edge & 1)) || (M::a(k) == 1 && (edge & 2)) ||
+                                             (M::b(k) == -1 && (edge & 4)) || (M::b(k) == 1 && (edge & 8)));
                 int to = 0;
                 if (M::a(k) == 1) to += dA_p; else if (M::a(k) == -1) to += dA_m;
                 if (M::b(k) == 1) to += dB_p; else if (M::b(k) == -1) to += dB_m;
                 if (M::m(k) == 1) to += dM_p; else if (M::m(k) == -1) to += dM_m;
-                // opposite directions share a weight, so the FP16 shift of slot ko is w_k ref
-                const R wk = R(V::w(k));
                 const unsigned t = Store<S, R>::kStochastic ? pair_word(nbits, k) : 0u;
                 const long long off = bounce ? (long long)(opposite(k) - k) * (long long)nn : (long long)to;
-                if constexpr (kSh) Store<S, R>::store2_raw(dk + 2 * off, 0, fo, ho, t);
-                else Store<S, R>::store2(dk + 2 * off, 0, fo, ho, wk * p->rho_ref, wk * p->E_ref, t);
-                dk += 2 * nn;
-            };
-            emit(0, R(V::w(0)) * KN, R(V::w(0)) * KG, fvk(0), hvk(0));
-            constexpr double w1 = V::w(1);
-            R kn = R(w1) * KN, kg = R(w1) * KG;
-            R pn = R(4.5 * w1) * PN, qn = R(4.5 * w1) * rho, pg = R(4.5 * w1) * PG, qg = R(4.5 * w1) * E_pf;
-            R rn = R(3.0 * w1) * PN, sn = R(3.0 * w1) * rho, rg = R(3.0 * w1) * PG, sg = R(3.0 * w1) * E_pf;
-#pragma unroll
-            for (int k = 1; k < Q; k += 2) {
-                if (k == (Q == 19 ? 7 : 5)) {   // first next-nearest direction
-                    const R h = R(V::w(Q - 1) / w1);
-                    kn *= h; kg *= h; pn *= h; qn *= h; pg *= h; qg *= h; rn *= h; sn *= h; rg *= h; sg *= h;
-                }
-                // s = c_k.u and t = c_k.v, each summed from its first term
-                R s = R(0), t = R(0);
-                bool first = true;
-                auto add = [&](int cc, R x, R y) {
-                    if (cc == 0) return;
-                    const R xs = cc > 0 ? x : -x, ys = cc > 0 ? y : -y;
-                    s = first ? xs : s + xs;
-                    t = first ? ys : t + ys;
-                    first = false;
-                };
-                add(M::a(k), u[0], v[0]);
-                add(M::b(k), u[1], v[1]);
-                add(M::m(k), u[2], v[2]);
-                const R s2 = s * s, t2 = t * t;
-                const R aE = fma(pn, s2, fma(qn, t2, kn)), bE = fma(pg, s2, fma(qg, t2, kg));
-                const R aO = fma(rn, s, sn * t), bO = fma(rg, s, sg * t);
-                emit(k, aE + aO, bE + bO, fvk(k), hvk(k));
-                emit(k + 1, aE - aO, bE - bO, fvk(k + 1), hvk(k + 1));
-            }
+                store_pop(dk + off, 0, v, t);
+                dk += nn;
+            });
         };
-        if (wall_lo || wall_hi || edge) collide(std::true_type{});
+        if (gu || gd || edge) collide(std::true_type{});
         else collide(std::false_type{});
     }
 };
@@ -628,49 +426,58 @@ __device__ __forceinline__ void fused_tile(const S* __restrict__ src, S* __restr
         }
     };
 
+    using Slots = typename St::Slots;
     if (tid >= NC) {
         // producers: iteration i builds M(i) and F(i-1).  M(i) and F(i-1)
         // overwrite the buffers that C(i-4) read last.
         // SPLIT: from plane zb + 3 on the consumers form the tile's moments
         // and the producers the border's.
         const int t = tid - NC;
+        int plane = wrapi(zb - 2, G.nm);   // wrapped index of plane i
         for (int i = zb - 2; i < ze + 3; ++i) {
             const int cw = i - 4;
             if (cw >= zb && cw < ze) wait(empty, cw - zb);
             const bool m_need = i <= ze + 1 && (walls ? (i >= 0 && i < G.nm) : true);
             const bool split = SPLIT && i >= zb + 3 && i <= ze + 1;
             if (m_need) {
-                if (split) st.m_border(i, t, NP);
-                else st.m_stage(i, t, NP);
+                const Slots sm(i);
+                if (split) st.m_border(sm, plane * st.plane_n, t, NP);
+                else st.m_stage(sm, plane * st.plane_n, t, NP);
             }
             if (split) wait(mint, i - zb - 3);
             asm volatile("bar.sync 1, %0;" ::"r"(NP));
             const int f = i - 1;
             const bool f_need = f >= zb - 1 && f <= ze && (walls ? (f >= 0 && f < G.nm) : true);
-            if (f_need) st.f_stage(f, t, NP);
+            if (f_need) st.f_stage(Slots(f), t, NP);
             asm volatile("bar.sync 1, %0;" ::"r"(NP));
             bool withhold = false;
             if constexpr (FAULT) withhold = i == fault_plane && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
             if (t == 0 && !withhold) mbar_arrive(full + ((i - zb + 2) % D));
+            plane = plane + 1 == G.nm ? 0 : plane + 1;
         }
     } else {
         // consumers: C(c) needs M(c+2) and F(c+1), i.e. producer iteration c+2
         const int ta = tid % TX, tb = tid / TX;
         const int ga = a0 + ta, gb = b0 + tb;
         const bool owns = ga < G.na && gb < G.nb;
-        const int n_ab = gb * G.na + ga;
         const int dA_m = ga == 0 ? G.na - 1 : -1, dA_p = ga == G.na - 1 ? 1 - G.na : 1;
         const int dB_m = (gb == 0 ? G.nb - 1 : -1) * G.na, dB_p = (gb == G.nb - 1 ? 1 - G.nb : 1) * G.na;
         const int edge = XW ? wall_edges(*p, Q, ga, gb, G.na, G.nb) : 0;
+        // the thread's own ring node: its column of a plane and ring indices
+        const int ring_n = st.ring_b[tb + Sh::RB] + st.ring_a[ta + 2];
+        const int ring_r = (tb + Sh::RB) * Sh::RW + ta + 2, ring_f = (tb + Sh::FB) * Sh::FW + ta + 1;
+        int ahead = wrapi(zb + 3, G.nm);   // wrapped index of plane c + 3
         for (int c = zb; c < ze; ++c) {
             wait(full, c - zb + 4);
+            const Slots sl(c);
             if (SPLIT && c + 3 <= ze + 1) {
-                const int m = c + 3;
-                if (walls ? m < G.nm : true) st.m_interior(m, ta, tb);
+                if (walls ? c + 3 < G.nm : true)
+                    st.template m_node<kUseKeep>(ahead * st.plane_n + ring_n, sl.phi_at(0), sl.rut_at(3), ring_r, ring_f);
                 mbar_arrive(mint + ((c - zb) % D));
             }
-            if (owns) st.template c_stage<XW>(c, ta, tb, n_ab, dA_m, dA_p, dB_m, dB_p, edge, cnt);
+            if (owns) st.template c_stage<XW>(sl, ring_f, ring_n, dA_m, dA_p, dB_m, dB_p, edge, cnt);
             mbar_arrive(empty + ((c - zb) % D));
+            ahead = ahead + 1 == G.nm ? 0 : ahead + 1;
         }
     }
 }

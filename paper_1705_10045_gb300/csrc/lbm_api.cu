@@ -217,6 +217,12 @@ void lbm_default_params(lbm_params* p) {
 
 int lbm_create(const lbm_params* p, lbm_handle** out) {
     lbm::TraceRange trace_("lbm_create");
+    return lbm::create_handle(p, out, true);
+}
+
+}  // extern "C"
+
+int lbm::create_handle(const lbm_params* p, lbm_handle** out, bool phases) {
     if (!p || !out) {
         set_error("lbm_create: null argument");
         return LBM_ERR_INVALID_ARG;
@@ -296,9 +302,16 @@ int lbm_create(const lbm_params* p, lbm_handle** out) {
         lbm_destroy(h);
         return rc;
     }
+    const size_t extb = h->Q == 9 ? lbm::Backend<9>::phase_bytes(p->storage) : lbm::Backend<19>::phase_bytes(p->storage);
+    if (phases && extb && p->step_kernel == LBM_STEP_FUSED && cudaMalloc(&h->ext, extb * (size_t)h->nn) != cudaSuccess) {
+        h->ext = nullptr;
+        (void)cudaGetLastError();   // a refused allocation is not an error of the handle
+    }
     *out = h;
     return LBM_OK;
 }
+
+extern "C" {
 
 int lbm_coexistence(double T, double* rho_v, double* rho_l) {
     if (!rho_v || !rho_l || !lbm::coexistence(T, rho_v, rho_l)) {
@@ -616,6 +629,7 @@ void lbm_destroy(lbm_handle* h) {
     cudaFree(h->pop[0]);
     cudaFree(h->pop[1]);
     cudaFree(h->fld);
+    cudaFree(h->ext);
     cudaFree(h->cnt);
     cudaFree(h->partials);
     cudaFree(h->staging);

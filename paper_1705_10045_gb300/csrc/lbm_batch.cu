@@ -237,7 +237,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_params* p, const double* rho, const do
     q.device = b->common.device;
     q.step_kernel = LBM_STEP_FUSED;
     lbm_handle* h = nullptr;
-    if (int rc = lbm_create(&q, &h)) return rc;
+    if (int rc = lbm::create_handle(&q, &h, false)) return rc;
     if (int rc = lbm_init(h, rho, u, eps, mem)) {
         lbm_destroy(h);
         return rc;

@@ -121,12 +121,11 @@ template <typename S, typename R, bool WALL> struct Strip {
             const R inv_rho = R(1) / o.rho;
             rho[J] = o.rho;
             E[J] = o.E;
-            T[J] = o.E / (o.rho * p.c_v);
+            T[J] = Math::temperature(p, o.rho, inv_rho, o.E);
             ua[J] = o.ja * inv_rho;
             um[J] = o.jm * inv_rho;
-            P[J] = eos_pressure(p, o.rho, T[J]);
-            const R U = ::fma(-o.rho, R(1.0 / 3.0), P[J]);
-            phi[J] = U < R(0) ? sqrt(-U) : R(0);
+            P[J] = Math::pressure(p, o.rho, T[J]);
+            phi[J] = Math::phi_of(Math::potential(o.rho, P[J]));
         }
         phl[J] = __shfl_up_sync(0xffffffffu, phi[J], 1);
         phr[J] = __shfl_down_sync(0xffffffffu, phi[J], 1);
@@ -142,7 +141,7 @@ template <typename S, typename R, bool WALL> struct Strip {
         const R u[3] = {hi ? phl[J] : phl[U], hi ? phi[J] : phi[U], hi ? phr[J] : phr[U]};
         const R o[3] = {phl[J], phi[J], phr[J]};
         R du[3];
-        Math::force(p, [&](int a, int, int m) { return m < 0 ? d[a + 1] : (m > 0 ? u[a + 1] : o[a + 1]); }, rho[J], du);
+        Math::force(p, [&](int a, int, int m) { return m < 0 ? d[a + 1] : (m > 0 ? u[a + 1] : o[a + 1]); }, rho[J], R(0), du);
         da[J] = du[0];
         dm[J] = du[2];
     }
@@ -160,33 +159,29 @@ template <typename S, typename R, bool WALL> struct Strip {
             if (edge & 1) ud = -us;
         }
         const R own_m = -::fma(dm[J], half, um[J]);
-        R div = R(0), cond = R(0);
-        Math::diff_div(uu, ud, div);
-        Math::diff_div(gu ? own_m : ::fma(dm[U], half, um[U]), gd ? own_m : ::fma(dm[D], half, um[D]), div);
+        typename Math::Axis ax[2] = {{uu, ud, Tc, Tc, r, r},
+                                     {gu ? own_m : ::fma(dm[U], half, um[U]), gd ? own_m : ::fma(dm[D], half, um[D]), Tc,
+                                      Tc, r, r}};
         if (p.conduction) {
-            R Tu = __shfl_down_sync(0xffffffffu, Tc, 1), Td = __shfl_up_sync(0xffffffffu, Tc, 1);
-            R ru = r, rd = r;
+            ax[0].Tu = __shfl_down_sync(0xffffffffu, Tc, 1);
+            ax[0].Td = __shfl_up_sync(0xffffffffu, Tc, 1);
+            // T beyond a wall: mirrored, or reflected about the wall temperature
+            ax[1].Tu = gu ? (p.T_fixed_hi ? R(2) * p.T_hi - Tc : Tc) : T[U];
+            ax[1].Td = gd ? (p.T_fixed_lo ? R(2) * p.T_lo - Tc : Tc) : T[D];
+            if (WALL && (edge & 2)) ax[0].Tu = p.T_fixed_x[1] ? R(2) * p.T_x[1] - Tc : Tc;
+            if (WALL && (edge & 1)) ax[0].Td = p.T_fixed_x[0] ? R(2) * p.T_x[0] - Tc : Tc;
             if (p.chi_mode) {
-                ru = __shfl_down_sync(0xffffffffu, r, 1);
-                rd = __shfl_up_sync(0xffffffffu, r, 1);
+                ax[0].ru = __shfl_down_sync(0xffffffffu, r, 1);
+                ax[0].rd = __shfl_up_sync(0xffffffffu, r, 1);
+                if (WALL && (edge & 2)) ax[0].ru = r;
+                if (WALL && (edge & 1)) ax[0].rd = r;
+                if (!gu) ax[1].ru = rho[U];
+                if (!gd) ax[1].rd = rho[D];
             }
-            if (WALL && edge) {   // T mirrored or reflected about the wall temperature
-                if (edge & 2) { Tu = p.T_fixed_x[1] ? R(2) * p.T_x[1] - Tc : Tc; ru = r; }
-                if (edge & 1) { Td = p.T_fixed_x[0] ? R(2) * p.T_x[0] - Tc : Tc; rd = r; }
-            }
-            const R half_lc = conductivity(p, r) * half;
-            Math::diff_cond(Tc, Tu, Td, half_lc, conductivity(p, ru), conductivity(p, rd), cond);
-            Tu = gu ? (p.T_fixed_hi ? R(2) * p.T_hi - Tc : Tc) : T[U];
-            Td = gd ? (p.T_fixed_lo ? R(2) * p.T_lo - Tc : Tc) : T[D];
-            Math::diff_cond(Tc, Tu, Td, half_lc, conductivity(p, gu ? r : rho[U]), conductivity(p, gd ? r : rho[D]),
-                            cond);
         }
         if (!owns) return;
-        R dE = R(0);
-        if (p.pressure_work) dE += -P[J] * div;
-        if (p.conduction) dE += cond;
-        if (p.latent != R(0)) dE += latent_heat(p, r, Tc, div);
-        const bool clamp = ::fma(-r, R(1.0 / 3.0), P[J]) >= R(0), bad = !(finite_pos(r) && finite_pos(E[J]));
+        const R dE = Math::energy_change(p, r, Tc, P[J], ax, 2);
+        const bool clamp = Math::potential(r, P[J]) >= R(0), bad = !(Math::positive(r) && Math::positive(E[J]));
         if (clamp || bad) {
             if (clamp) atomicAdd(&cnt->clamps, 1ull);
             if (bad) atomicAdd(&cnt->bad, 1ull);
