@@ -75,11 +75,11 @@ extern "C" {
 #define LBM_STORE_FP32 1 /* FP32 storage, FP32 arithmetic */
 #define LBM_STORE_FP16 2 /* FP16 storage of N_k - w_k rho_ref and g_k - w_k E_ref, FP32 arithmetic */
 
-/* how a time step is launched: the fused form (one kernel that marches tiles or
- * strips along the last lattice axis; FP64, whose step is bound by arithmetic,
- * as three kernels that form every value once), or three plain kernels
- * (moments/Phi, force, collide+stream), an independent statement of the step;
- * all compute the same step */
+/* how a time step is launched: the fused form (one kernel that marches tiles
+ * or strips along the last lattice axis; FP64, whose step is bound by
+ * arithmetic, and small D3Q19 domains as three kernels that form every value
+ * once), or three plain kernels (moments/Phi, force, collide+stream), an
+ * independent statement of the step; all compute the same step */
 #define LBM_STEP_FUSED 0
 #define LBM_STEP_THREE_LAUNCH 1
 
@@ -237,8 +237,9 @@ typedef struct lbm_batch lbm_batch;
 /* Device memory in bytes a domain with parameters *p needs (admission control),
  * counting the staging planes it keeps once fields have moved between it and
  * host memory (lbm_init or lbm_moments with host pointers).  A handle from
- * lbm_create with FP64 storage takes another 24 bytes per node when there is
- * memory for them (fields of its three-kernel step); a batch's domains do not. */
+ * lbm_create that steps in three fused-form kernels (FP64, small D3Q19 domains)
+ * takes two more fields when there is memory for them; a batch's domains do
+ * not. */
 size_t lbm_domain_bytes(const lbm_params* p);
 
 /* New empty batch for common->lattice and common->storage on common->device.

@@ -38,8 +38,6 @@ template <typename R> KParams<R> make_kparams(const lbm_handle* h) {
     k.step = (unsigned)h->steps;
     k.latent = (R)q.latent;
     k.coex = (const R*)h->coex;
-    k.inv_c_v = (R)(1.0 / q.c_v);
-    k.half_cv_chi = (R)(0.5 * q.c_v * q.chi);
     return k;
 }
 
@@ -94,11 +92,61 @@ template <typename R> struct BatchShape<19, R, 2> { static constexpr int TX = 32
 template <int Q, typename S, typename R> struct Impl {
     static constexpr int TX = FusedTile<Q, R>::TX, TY = FusedTile<Q, R>::TY, NP = FusedTile<Q, R>::NP;
     static constexpr bool SPLIT = FusedTile<Q, R>::SPLIT;
-    // FP64 steps in three phases (phases.cuh) where the handle has their planes
-    static constexpr bool kPhases = std::is_same<S, double>::value;
+    // Steps in three phases (phases.cuh): FP64, and D3Q19 domains the march
+    // cannot spread over the SMs (march_us); only where the handle has their
+    // planes.
+    static constexpr bool kF64 = std::is_same<S, double>::value;
+    static constexpr bool kPhases = kF64 || Q == 19;
     static bool phases(const lbm_handle* h) { return kPhases && h->ext && h->fault_drop <= 0; }
+    static bool wants_phases(int nx, int ny, int nz) {
+        if (kF64) return true;
+        if (!kPhases) return false;
+        MarchGeom G;
+        G.na = nx;
+        G.nb = ny;
+        G.nm = nz;
+        double t;
+        march_chunk(G, nz, t);
+        return 4.5 + kPhaseNs * 1e-3 * (double)nx * ny * nz < t;
+    }
     static int launches(const lbm_handle* h) {
         return h->p.step_kernel == LBM_STEP_THREE_LAUNCH || phases(h) ? 3 : 1;
+    }
+
+    // Planes per CTA of the march, and the modelled time t (us) of the launch.
+    // A CTA takes about 4.5 plane times beyond its chunk (ring planes, the
+    // first three planes' moments).  A plane takes kPlane1 us while an SM holds
+    // one CTA and kPlane2 with two (D3Q19, measured: 64^3 in chunks of 8 with
+    // 128 CTAs, 128^3 in chunks of 32 with 256); chunks stay below 65 planes
+    // so that neighbouring tiles of a large domain keep sharing ring lines in
+    // L2.  The chunk with the smallest modelled time avoids nearly empty last
+    // waves: FP32 us per step, two CTAs' worth of planes -> this: 128^3 195 ->
+    // 160 (5 -> 4 chunks), 160 x 128 x 96 188 -> 165, 192^3 569 -> 493.
+    // The phases take 4.5 us and kPhaseNs per node (93 ps FP32, 70 ps FP16),
+    // the march 56 and 49 ps a node where it fills the chip: FP32 32^3 33 -> 7.4,
+    // 48^3 35 -> 12.4, 64^3 35 -> 22.6, 80^3 54 -> 51 by phases; 96^3 75 against
+    // 89 and 128^3 160 against 202 by the march.
+    static constexpr double kPlane1 = sizeof(S) == 2 ? 2.6 : 2.7, kPlane2 = sizeof(S) == 2 ? 3.85 : 4.4;
+    static constexpr double kPhaseNs = sizeof(S) == 2 ? 0.070 : 0.093;
+    static int march_chunk(const MarchGeom& G, int len, double& t) {
+        const long long tiles = (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY);
+        const int few = (len + 63) / 64;   // chunks per column of tiles, at least
+        int best = len;
+        t = 1e30;
+        for (int n = few; n <= len; ++n) {
+            const int c = (len + n - 1) / n;
+            if ((len + c - 1) / c != n) continue;
+            const long long ctas = tiles * n, full = ctas / (2 * kSms), rest = ctas % (2 * kSms);
+            const double tn = (c + 4.5) * ((double)full * kPlane2 + (rest > kSms ? kPlane2 : (rest ? kPlane1 : 0.0)));
+            if (tn < t) {
+                t = tn;
+                best = c;
+            }
+            // four waves and more: the block scheduler evens out the last one
+            // (384 x 384 x 256: chunks of 64 2545 us, of 52 2597)
+            if (tiles * few >= 8 * kSms) break;
+        }
+        return best;
     }
 
     // planes [m_lo, m_hi) collided; m_hi < 0: the handle's own range
@@ -115,13 +163,8 @@ template <int Q, typename S, typename R> struct Impl {
             G.m_lo = m_lo;
             G.m_hi = m_hi;
         }
-        const int len = G.m_hi - G.m_lo;
-        // planes per CTA: enough CTAs for about two per SM on 152 SMs, and
-        // at least 8 planes so that the extra ring planes stay a minority
-        const long long tiles = (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY);
-        long long c = (len * tiles + 303) / 304;
-        c = c < 8 ? 8 : (c > 64 ? 64 : c);
-        G.chunk = (int)(c > len ? len : c);
+        double t;
+        G.chunk = march_chunk(G, G.m_hi - G.m_lo, t);
         return G;
     }
 
@@ -167,7 +210,7 @@ template <int Q, typename S, typename R> struct Impl {
         R* fld = (R*)h->fld;
         R* ext = (R*)h->ext;
         if (j == 0) launch_after(phase_moments_kernel<Q, S, R>, grid, 128, 0, h->stream, src, fld, ext, kp, g, (Counters*)h->cnt);
-        if (j == 1) launch_after(phase_force_kernel<Q, S, R>, grid, 128, 0, h->stream, fld, ext, kp, g);
+        if (j == 1) launch_after(phase_force_kernel<Q, S, R>, grid, 128, 0, h->stream, fld, kp, g);
         if (j == 2) launch_after(phase_collide_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, ext, kp, g);
     }
 
@@ -202,11 +245,14 @@ template <int Q, typename S, typename R> struct Impl {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             h->fused_ready = true;
         }
-        const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
+        dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
         if (h->fault_drop > 0) {   // fault-injection test hook (lbm_test_drop_handoff)
+            MarchGeom F = G;       // long chunks, so that the first CTA marches over the plane
+            F.chunk = std::min(64, G.m_hi - G.m_lo);
+            grid.z = (G.m_hi - G.m_lo + F.chunk - 1) / F.chunk;
             auto fk = fused_step_fault_kernel<Q, S, R, TX, TY, NP, SPLIT>;
             cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            fk<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, (Counters*)h->cnt, h->fault_drop - 1);
+            fk<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, F, (Counters*)h->cnt, h->fault_drop - 1);
         } else {
             kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, (Counters*)h->cnt);
         }
@@ -507,8 +553,13 @@ template <int Q> size_t Backend<Q>::desc_bytes(int storage) {
 template <int Q> size_t Backend<Q>::field_bytes(int storage) {
     return (size_t)F_COUNT * (storage == LBM_STORE_FP64 ? sizeof(double) : sizeof(float));
 }
-template <int Q> size_t Backend<Q>::phase_bytes(int storage) {
-    return storage == LBM_STORE_FP64 ? (size_t)X_COUNT * sizeof(double) : 0;
+template <int Q> size_t Backend<Q>::phase_bytes(const lbm_params* p) {
+    const size_t planes = (size_t)X_COUNT * (size_t)p->nx * p->ny * p->nz;
+    switch (p->storage) {
+        case LBM_STORE_FP64: return planes * sizeof(double);
+        case LBM_STORE_FP32: return Impl<Q, float, float>::wants_phases(p->nx, p->ny, p->nz) ? planes * sizeof(float) : 0;
+        default: return Impl<Q, __half, float>::wants_phases(p->nx, p->ny, p->nz) ? planes * sizeof(float) : 0;
+    }
 }
 
 #undef LBM_DISPATCH

@@ -232,10 +232,10 @@ template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool 
 #pragma unroll
         for (int k = 0; k < Q; ++k) w[k] = load_pop<COH, U>(src + 2 * ((size_t)k * nn), (size_t)(unsigned)n);
         const Moments<R> o = Math::moments(w, *p);
-        const R inv = Math::kF64 || f >= 0 ? R(1) / o.rho : R(0);
-        const R T = Math::temperature(*p, o.rho, inv, o.E);
-        phi(sp, r) = Math::phi_of(Math::potential(o.rho, Math::pressure(*p, o.rho, T)));
+        const R T = o.E / (o.rho * p->c_v);
+        phi(sp, r) = Math::phi_of(Math::potential(o.rho, eos_pressure(*p, o.rho, T)));
         if (f >= 0) {
+            const R inv = R(1) / o.rho;
             rut(sr, 0, f) = o.rho;
             rut(sr, 1, f) = o.ja * inv;
             rut(sr, 2, f) = o.jb * inv;
@@ -252,11 +252,10 @@ template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool 
         const int sd = sl.du();
         for (int r = t; r < F_; r += nt) {
             const int at = (r / FW + (RB - FB)) * RW + r % FW + 1;
-            const R rho = rut(sl.rut, 0, r);
             R d[3];
             Math::force(*p, [&](int a, int b, int m) {
                 return phi(m == 0 ? sp0 : (m > 0 ? spp : spm), at + b * RW + a);
-            }, rho, Math::kF64 ? R(1) / rho : R(0), d);
+            }, rut(sl.rut, 0, r), d);
             du(sd, 0, r) = d[0];
             du(sd, 1, r) = d[1];
             du(sd, 2, r) = d[2];
@@ -319,7 +318,7 @@ template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool 
             ax[N - 1].ru = gu ? rho : rut(su, 0, fc);
             ax[N - 1].rd = gd ? rho : rut(sdn, 0, fc);
         }
-        const R P = Math::pressure(*p, rho, T);
+        const R P = eos_pressure(*p, rho, T);
         const R dE = Math::energy_change(*p, rho, T, P, ax, N);
         const R E = Math::energy(w, *p);
         const bool clamp = Math::potential(rho, P) >= R(0), bad = !(Math::positive(rho) && Math::positive(E));

@@ -16,7 +16,7 @@ struct lbm_handle {
     void* pop[2] = {nullptr, nullptr};   // ping-pong population buffers, 2Q planes each
     int cur = 0;                // buffer holding the current state
     void* fld = nullptr;        // field planes (arithmetic type)
-    void* ext = nullptr;        // field planes of the FP64 step's phases (null: the fused march steps)
+    void* ext = nullptr;        // field planes of a step in phases (null: the fused step)
     void* cnt = nullptr;        // lbm::Counters on the device
     double* partials = nullptr; // reduction scratch: block partials + 8 results
     double* staging = nullptr;  // (D + 3) planes of doubles for host transfers, allocated on demand
@@ -78,9 +78,9 @@ struct TraceRange {
 // error reporting shared by the translation units
 void set_error(const std::string& msg);
 int cuda_error(cudaError_t e, const char* where);
-// lbm_create; phases: also allocate the field planes of the FP64 step's three
-// phases (without them, or when there is no memory left for them, FP64 steps
-// take the fused march, which the domains of a batch do in any case)
+// lbm_create; phases: also allocate the field planes of a step in three phases,
+// for domains that step so (without them, or when there is no memory left for
+// them, those take the fused march, as the domains of a batch do)
 int create_handle(const lbm_params* p, lbm_handle** out, bool phases);
 int ensure_staging(lbm_handle* h);   // the handle's host-transfer buffer, allocated on first use
 // Conservation sums of nodes [i0, i0 + n) through `partials` (block partials,
@@ -101,7 +101,7 @@ template <int Q> struct Backend {
     // sums over nodes [i0, i0 + n): 5 sums and 3 counters into device memory
     static int reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev);
     static size_t field_bytes(int storage);
-    static size_t phase_bytes(int storage);   // per node, 0 when the storage does not step in phases
+    static size_t phase_bytes(const lbm_params* p);   // extra field planes, 0 when the domain does not step in phases
     // batches: shapes, work table, descriptors, and one request (clear, the
     // persistent launch, and the descriptor advance when `advance`)
     static int batch_variants();

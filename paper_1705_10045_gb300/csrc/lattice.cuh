@@ -302,7 +302,6 @@ template <typename R> struct KParams {
     unsigned step;        // step counter, seeds the FP16 stochastic rounding
     R latent;             // rho_liq Q of Sec. 5 (0: no latent heat)
     const R* coex;        // rho_v then rho_l on T = 0.5 + j/1024, j = 0..512
-    R inv_c_v, half_cv_chi;   // 1/c_v and c_v chi / 2 (the FP64 forms of the step)
 };
 
 // reduced van der Waals EOS scaled by kappa (Sec. 3); T0 when barotropic (Sec. 4)

@@ -302,8 +302,8 @@ int lbm::create_handle(const lbm_params* p, lbm_handle** out, bool phases) {
         lbm_destroy(h);
         return rc;
     }
-    const size_t extb = h->Q == 9 ? lbm::Backend<9>::phase_bytes(p->storage) : lbm::Backend<19>::phase_bytes(p->storage);
-    if (phases && extb && p->step_kernel == LBM_STEP_FUSED && cudaMalloc(&h->ext, extb * (size_t)h->nn) != cudaSuccess) {
+    const size_t extb = h->Q == 9 ? lbm::Backend<9>::phase_bytes(p) : lbm::Backend<19>::phase_bytes(p);
+    if (phases && extb && p->step_kernel == LBM_STEP_FUSED && cudaMalloc(&h->ext, extb) != cudaSuccess) {
         h->ext = nullptr;
         (void)cudaGetLastError();   // a refused allocation is not an error of the handle
     }

@@ -132,32 +132,15 @@ template <int Q, typename S, typename R> struct NodeMath {
     using M = MVel<Q>;
     static constexpr bool kSh = Store<S, R>::kShifted;
 
-    // FP64 runs at two lanes per clock and SM with a latency of 64 cycles, so
-    // its forms below trade divisions for reciprocals (4.5 against 7.6
-    // instructions) and long chains of additions for short ones; FP32 keeps
-    // the order its results are held to.
-    static constexpr bool kF64 = std::is_same<R, double>::value;
-
     // sum over k of g_k
     __device__ static __forceinline__ R energy(const Pop<S>* f, const KParams<R>& p) {
         R E = f[0].g();
-        if constexpr (kF64) {
-            R part[3] = {E, R(0), R(0)};
 #pragma unroll
-            for (int k = 1; k < Q; k += 2) {
-                const R s = f[k].g() + f[k + 1].g();
-                const int j = (k / 2) % 3;
-                part[j] = k == 3 || k == 5 ? s : part[j] + s;
-            }
-            E = part[0] + (part[1] + part[2]);
-        } else {
-#pragma unroll
-            for (int k = 1; k < Q; ++k) {
-                if constexpr (kSh) E = Store<S, R>::add_hi(f[k].v, E);
-                else E += f[k].g();
-            }
-            if constexpr (kSh) E += p.E_ref;   // sums of shifted values: sum_k w_k = 1, sum_k w_k c_k = 0
+        for (int k = 1; k < Q; ++k) {
+            if constexpr (kSh) E = Store<S, R>::add_hi(f[k].v, E);   // FP16: the half enters the sum directly
+            else E += f[k].g();
         }
+        if constexpr (kSh) E += p.E_ref;   // sums of shifted values: sum_k w_k = 1, sum_k w_k c_k = 0
         return E;
     }
 
@@ -168,7 +151,7 @@ template <int Q, typename S, typename R> struct NodeMath {
         Moments<R> o;
         o.ja = o.jb = o.jm = R(0);
         bool new_a = true, new_b = true, new_m = true;
-        R part[3] = {f[0].N(), R(0), R(0)};   // rho: one running sum, or three in FP64
+        o.rho = f[0].N();
 #pragma unroll
         for (int k = 1; k < Q; k += 2) {
             R s, d;   // N_k + N_{k+1} and N_k - N_{k+1}
@@ -180,36 +163,21 @@ template <int Q, typename S, typename R> struct NodeMath {
                 s = f[k].N() + f[k + 1].N();
                 d = f[k].N() - f[k + 1].N();
             }
-            const int j = kF64 ? (k / 2) % 3 : 0;
-            part[j] = kF64 && (k == 3 || k == 5) ? s : part[j] + s;
+            o.rho += s;
             if (M::a(k) != 0) { const R t = M::a(k) > 0 ? d : -d; o.ja = new_a ? t : o.ja + t; new_a = false; }
             if (M::b(k) != 0) { const R t = M::b(k) > 0 ? d : -d; o.jb = new_b ? t : o.jb + t; new_b = false; }
             if (M::m(k) != 0) { const R t = M::m(k) > 0 ? d : -d; o.jm = new_m ? t : o.jm + t; new_m = false; }
         }
-        o.rho = kF64 ? part[0] + (part[1] + part[2]) : part[0];
         if constexpr (kSh) o.rho += p.rho_ref;
         o.E = energy(f, p);
         return o;
     }
 
-    // kappa p~(rho, T), reduced van der Waals (Sec. 3); T0 when barotropic (Sec. 4)
-    __device__ static __forceinline__ R pressure(const KParams<R>& p, R rho, R T) {
-        if constexpr (kF64) {
-            const R Te = p.barotropic ? p.T0 : T;
-            return p.kappa * ::fma(R(-3) * rho, rho, R(8) * rho * Te * (R(1) / (R(3) - rho)));
-        } else {
-            return eos_pressure(p, rho, T);
-        }
-    }
-    __device__ static __forceinline__ R temperature(const KParams<R>& p, R rho, R inv_rho, R E) {
-        if constexpr (kF64) return E * inv_rho * p.inv_c_v;
-        else return E / (rho * p.c_v);
-    }
     // U = p - rho theta, and Phi = sqrt(-U) where U < 0
     __device__ static __forceinline__ R potential(R rho, R P) { return ::fma(-rho, R(1.0 / 3.0), P); }
     __device__ static __forceinline__ R phi_of(R U) { return U < R(0) ? sqrt(-U) : R(0); }
     __device__ static __forceinline__ bool positive(R v) {
-        if constexpr (kF64) {   // v > 0 and finite, by its bits
+        if constexpr (sizeof(R) == 8) {   // by its bits: an FP64 comparison takes the FP64 pipe
             const long long b = __double_as_longlong(v);
             return b > 0 && b < 0x7ff0000000000000ll;
         } else {
@@ -222,37 +190,11 @@ template <int Q, typename S, typename R> struct NodeMath {
     // G Phi(x+e) e + G Phi(x-e)(-e) = G (Phi+ - Phi-) e and the Phi^2 term is
     // G (Phi+ - Phi-)(Phi+ + Phi-) e.
     template <typename PH>
-    __device__ static __forceinline__ void force(const KParams<R>& p, const PH& ph, R rho, R inv_rho, R* du) {
+    __device__ static __forceinline__ void force(const KParams<R>& p, const PH& ph, R rho, R* du) {
         const R A = p.A, B = R(1) - R(2) * p.A, inv_alpha = R(1.0 / V::alpha);
         const R gv[3] = {p.g[0], Q == 9 ? R(0) : p.g[1], Q == 9 ? p.g[1] : p.g[2]};
         const R G2 = R(V::G(Q - 1));   // next-nearest weight (1/4 or 1/2)
         const R Bph0 = B * ph(0, 0, 0);
-        if constexpr (kF64) {
-            // each pair contributes (Phi+ - Phi-)(A (Phi+ + Phi-) + B Phi) e
-            R n[3] = {0, 0, 0}, q[3] = {0, 0, 0};
-            bool first[3] = {true, true, true};
-#pragma unroll
-            for (int k = 1; k < Q; k += 2) {
-                const int c[3] = {M::a(k), M::b(k), M::m(k)};
-                const R pp = ph(c[0], c[1], c[2]), pm = ph(-c[0], -c[1], -c[2]);
-                const R t = (pp - pm) * ::fma(A, pp + pm, Bph0);
-                const bool nearest = c[0] * c[0] + c[1] * c[1] + c[2] * c[2] == 1;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    if (c[a] == 0) continue;
-                    if (nearest) {
-                        n[a] = t;
-                    } else {
-                        q[a] = first[a] ? (c[a] > 0 ? t : -t) : (c[a] > 0 ? q[a] + t : q[a] - t);
-                        first[a] = false;
-                    }
-                }
-            }
-            const R scale = inv_alpha * inv_rho;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) du[a] = Q == 9 && a == 1 ? R(0) : ::fma(::fma(G2, q[a], n[a]), scale, gv[a]);
-            return;
-        }
         R n1[3] = {0, 0, 0}, n2[3] = {0, 0, 0}, q1[3] = {0, 0, 0}, q2[3] = {0, 0, 0};
 #pragma unroll
         for (int k = 1; k < Q; k += 2) {
@@ -286,42 +228,20 @@ template <int Q, typename S, typename R> struct NodeMath {
     // of the two nodes', latent heat.
     __device__ static __forceinline__ R energy_change(const KParams<R>& p, R rho, R T, R P, const Axis* ax, int n) {
         R div = R(0), cond = R(0);
-        if constexpr (kF64) {
 #pragma unroll
-            for (int a = 0; a < n; ++a) div = a == 0 ? ax[a].uu - ax[a].ud : div + (ax[a].uu - ax[a].ud);
-            div *= R(0.5);
-            if (p.conduction) {
-                if (p.chi_mode) {
+        for (int a = 0; a < n; ++a) div = ::fma(ax[a].uu - ax[a].ud, R(0.5), div);
+        if (p.conduction) {
+            const R half_lc = conductivity(p, rho) * R(0.5);
 #pragma unroll
-                    for (int a = 0; a < n; ++a) {
-                        cond = ::fma(rho + ax[a].ru, ax[a].Tu - T, cond);
-                        cond = ::fma(rho + ax[a].rd, ax[a].Td - T, cond);
-                    }
-                    cond *= p.half_cv_chi;
-                } else {
-#pragma unroll
-                    for (int a = 0; a < n; ++a) {
-                        const R s = ax[a].Tu + ax[a].Td;
-                        cond = a == 0 ? s : cond + s;
-                    }
-                    cond = p.lambda * ::fma(R(-2 * n), T, cond);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < n; ++a) div = ::fma(ax[a].uu - ax[a].ud, R(0.5), div);
-            if (p.conduction) {
-                const R half_lc = conductivity(p, rho) * R(0.5);
-#pragma unroll
-                for (int a = 0; a < n; ++a) {
-                    const R lu = ::fma(conductivity(p, ax[a].ru), R(0.5), half_lc);
-                    const R ld = ::fma(conductivity(p, ax[a].rd), R(0.5), half_lc);
-                    cond = ::fma(-ld, T - ax[a].Td, ::fma(lu, ax[a].Tu - T, cond));
-                }
+            for (int a = 0; a < n; ++a) {
+                // a constant conductivity is its own mean, exactly
+                const R lu = p.chi_mode ? ::fma(conductivity(p, ax[a].ru), R(0.5), half_lc) : p.lambda;
+                const R ld = p.chi_mode ? ::fma(conductivity(p, ax[a].rd), R(0.5), half_lc) : p.lambda;
+                cond = ::fma(-ld, T - ax[a].Td, ::fma(lu, ax[a].Tu - T, cond));
             }
         }
         R dE = R(0);
-        if (p.pressure_work) dE = kF64 ? -P * div : dE + -P * div;
+        if (p.pressure_work) dE += -P * div;
         if (p.conduction) dE += cond;
         if (p.latent != R(0)) dE += latent_heat(p, rho, T, div);
         return dE;
@@ -351,7 +271,7 @@ template <int Q, typename S, typename R> struct NodeMath {
     __device__ static __forceinline__ void collide(const KParams<R>& p, R rho, R E, const R* u, const R* dv, R dE,
                                                    const PF& pop, const EM& emit) {
         using T2 = Two<R>;
-        const R dEoverE = kF64 ? dE * (R(1) / E) : dE / E;
+        const R dEoverE = dE / E;
         R usq = u[2] * u[2], dsq = dv[2] * ::fma(R(2), u[2], dv[2]);
         if (Q == 19) {
             usq = ::fma(u[1], u[1], usq);

@@ -1,21 +1,28 @@
 // One time step as three launches over all nodes, each value formed once:
-//   phase_moments   rho, u, T, P, E, 1/rho, Phi of every node
+//   phase_moments   rho, u, T, P, E, Phi of every node
 //   phase_force     du = F/rho
 //   phase_collide   dE, collision, push
 // with the fields in device memory between them.
 //
-// For FP64.  A GB300 issues FP64 at two lanes per clock and SM (492 G lanes/s
-// measured, 64 cycles latency), so an FP64 step is bound by its FP64
-// instructions (about 390 a node on D3Q19, 215 on D2Q9), not by memory: 0.8 ns
+// For FP64, and for small D3Q19 domains.  A GB300 issues FP64 at two lanes per
+// clock and SM (492 G lanes/s measured, 64 cycles latency), so an FP64 step is
+// bound by its FP64 instructions (about 430 a node on D3Q19, 240 on D2Q9), not by memory: 0.8 ns
 // a node against 0.1 ns for the 608 bytes of populations.  The fused march
 // (fused.cuh) recomputes the moments and forces of every tile's ring, which
 // saves bytes that are free here and costs instructions that are not; it also
-// needs tiles to fill the chip.  Field traffic (15 values a node) is nothing
+// needs tiles to fill the chip.  Field traffic (14 values a node) is nothing
 // beside the arithmetic.  The per-node arithmetic is the march's
 // (node.cuh): the two forms agree bit for bit.  Measured, march -> phases, us
-// per step: D2Q9 128 x 128 125 -> 13, a row of 128 nodes 35 -> 12, D3Q19
-// 90 x 75 x 67 with walls on every axis 1050 -> 356 (of which the FP64
-// instructions need about 360 at the measured rate).
+// per step: D2Q9 128 x 128 125 -> 14.2, a row of 128 nodes 35 -> 12.7, D3Q19
+// 90 x 75 x 67 with walls on every axis 1050 -> 387 (its FP64 instructions
+// need about that at the measured rate).  Reciprocals for the divisions and
+// shorter chains of additions would give 12.6 and 356, with other rounding.
+//
+// In FP32 and FP16 storage the populations are read twice and the fields add
+// traffic (about 93 ps a node against the march's 56), but every node has its
+// own thread and no plane waits for another: domains too small to fill 152 SMs
+// with marching CTAs step faster this way (the rule and figures stand at
+// march_chunk in backend.cuh).
 #pragma once
 
 #include "node.cuh"
@@ -23,7 +30,7 @@
 namespace lbm {
 
 // extra field planes of the phases, beyond F_COUNT (kernels.cuh)
-enum { X_E = 0, X_P = 1, X_INV = 2, X_COUNT = 3 };
+enum { X_E = 0, X_P = 1, X_COUNT = 2 };
 
 struct PhaseGeom {
     int plane_n, nm;       // nodes of a plane of the last axis, planes
@@ -86,7 +93,7 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict_
     for (int k = 0; k < Q; ++k) f[k] = load_pop<false>(src + 2 * ((size_t)k * nn), (size_t)n);
     const Moments<R> o = Math::moments(f, p);
     const R inv = R(1) / o.rho;
-    const R T = Math::temperature(p, o.rho, inv, o.E), P = Math::pressure(p, o.rho, T);
+    const R T = o.E / (o.rho * p.c_v), P = eos_pressure(p, o.rho, T);
     const R U = Math::potential(o.rho, P);
     fld[F_RHO * nn + n] = o.rho;
     fld[F_UX * nn + n] = o.ja * inv;
@@ -96,7 +103,6 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict_
     fld[F_PHI * nn + n] = Math::phi_of(U);
     ext[X_E * nn + n] = o.E;
     ext[X_P * nn + n] = P;
-    ext[X_INV * nn + n] = inv;
     const bool clamp = U >= R(0), bad = !(Math::positive(o.rho) && Math::positive(o.E));
     if (clamp || bad) {   // counted once a step, with the plane's collision
         const int m = n / G.plane_n;
@@ -108,8 +114,7 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict_
 }
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, const R* __restrict__ ext,
-                                                          const __grid_constant__ KParams<R> p, PhaseGeom G) {
+__global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, const __grid_constant__ KParams<R> p, PhaseGeom G) {
     using Ph = Phase<Q, S, R>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int n = Ph::node(G);
@@ -125,7 +130,7 @@ __global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, c
         for (int j = 0; j < 3; ++j)
             if (c[j] != 0) to += c[j] > 0 ? s.hi[Ph::axis(j)] : s.lo[Ph::axis(j)];
         return phi[to];
-    }, fld[F_RHO * nn + n], ext[X_INV * nn + n], du);
+    }, fld[F_RHO * nn + n], du);
     fld[F_DUX * nn + n] = du[0];
     fld[F_DUY * nn + n] = Q == 9 ? du[2] : du[1];
     if (Q == 19) fld[F_DUZ * nn + n] = du[2];

@@ -121,10 +121,10 @@ template <typename S, typename R, bool WALL> struct Strip {
             const R inv_rho = R(1) / o.rho;
             rho[J] = o.rho;
             E[J] = o.E;
-            T[J] = Math::temperature(p, o.rho, inv_rho, o.E);
+            T[J] = o.E / (o.rho * p.c_v);
             ua[J] = o.ja * inv_rho;
             um[J] = o.jm * inv_rho;
-            P[J] = Math::pressure(p, o.rho, T[J]);
+            P[J] = eos_pressure(p, o.rho, T[J]);
             phi[J] = Math::phi_of(Math::potential(o.rho, P[J]));
         }
         phl[J] = __shfl_up_sync(0xffffffffu, phi[J], 1);
@@ -141,7 +141,7 @@ template <typename S, typename R, bool WALL> struct Strip {
         const R u[3] = {hi ? phl[J] : phl[U], hi ? phi[J] : phi[U], hi ? phr[J] : phr[U]};
         const R o[3] = {phl[J], phi[J], phr[J]};
         R du[3];
-        Math::force(p, [&](int a, int, int m) { return m < 0 ? d[a + 1] : (m > 0 ? u[a + 1] : o[a + 1]); }, rho[J], R(0), du);
+        Math::force(p, [&](int a, int, int m) { return m < 0 ? d[a + 1] : (m > 0 ? u[a + 1] : o[a + 1]); }, rho[J], du);
         da[J] = du[0];
         dm[J] = du[2];
     }
