@@ -9,6 +9,7 @@
 #include "fused.cuh"
 #include "internal.h"
 #include "kernels.cuh"
+#include "output.cuh"
 #include "phases.cuh"
 #include "strip.cuh"
 
@@ -339,13 +340,14 @@ template <int Q, typename S, typename R> struct Impl {
                                                                            (Counters*)h->cnt);
         return cuda_error(cudaGetLastError(), "lbm_init launch");
     }
-    static int moments(lbm_handle* h, double* rho, double* u, double* T, double* P) {
+    template <typename O>
+    static int output(lbm_handle* h, O* rho, O* u, O* T, O* P, Counters* cnt_out) {
         const KParams<R> kp = make_kparams<R>(h);
         const unsigned g = grid_for(h->nn, 256);
         R* fld = (R*)h->fld;
-        fields_kernel<Q, S, R><<<g, 256, 0, h->stream>>>((const S*)h->pop[h->cur], fld, kp, (Counters*)h->cnt, 0);
-        force_kernel<Q, R><<<g, 256, 0, h->stream>>>(fld, kp);
-        output_kernel<Q, R><<<g, 256, 0, h->stream>>>(fld, kp, rho, u, T, P);
+        output_kernel<Q, S, R, O><<<g, 256, 0, h->stream>>>((const S*)h->pop[h->cur], fld, kp, rho, T, P, u != nullptr,
+                                                            (const Counters*)h->cnt, cnt_out);
+        if (u) output_velocity_kernel<Q, R, O><<<g, 256, 0, h->stream>>>(fld, kp, u);
         return cuda_error(cudaGetLastError(), "lbm_moments launch");
     }
     // ---- batches ---------------------------------------------------------
@@ -523,8 +525,12 @@ template <int Q> int Backend<Q>::launches(const lbm_handle* h) { LBM_DISPATCH(h,
 template <int Q> int Backend<Q>::init(lbm_handle* h, const double* rho, const double* u, const double* eps) {
     LBM_DISPATCH(h, init(h, rho, u, eps));
 }
-template <int Q> int Backend<Q>::moments(lbm_handle* h, double* rho, double* u, double* T, double* P) {
-    LBM_DISPATCH(h, moments(h, rho, u, T, P));
+template <int Q>
+int Backend<Q>::output(lbm_handle* h, const Outputs& o, Counters* cnt_out) {
+    if (o.single) {
+        LBM_DISPATCH(h, output(h, (float*)o.rho, (float*)o.u, (float*)o.T, (float*)o.P, cnt_out));
+    }
+    LBM_DISPATCH(h, output(h, (double*)o.rho, (double*)o.u, (double*)o.T, (double*)o.P, cnt_out));
 }
 template <int Q> int Backend<Q>::reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev) {
     LBM_DISPATCH(h, reduce(h, i0, n, partials, out_dev));

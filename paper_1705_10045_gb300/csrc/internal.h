@@ -20,6 +20,7 @@ struct lbm_handle {
     void* cnt = nullptr;        // lbm::Counters on the device
     double* partials = nullptr; // reduction scratch: block partials + 8 results
     double* staging = nullptr;  // (D + 3) planes of doubles for host transfers, allocated on demand
+    void* bounce = nullptr;     // pinned host buffer for small host outputs, allocated on demand
     void* coex = nullptr;       // coexistence table (arithmetic type) when p.latent != 0
     unsigned long long reported_bad = 0;
     long long steps = 0;
@@ -89,6 +90,14 @@ int ensure_staging(lbm_handle* h);   // the handle's host-transfer buffer, alloc
 int diagnose(lbm_handle* h, long long i0, long long n, double* partials, double out[8]);
 
 
+struct Counters;
+
+// the caller's output fields (any may be null), doubles or (single) floats
+struct Outputs {
+    void *rho, *u, *T, *P;
+    bool single;
+};
+
 // per-lattice entry points, dispatched on the storage format inside
 template <int Q> struct Backend {
     static int step(lbm_handle* h, int n);
@@ -97,7 +106,8 @@ template <int Q> struct Backend {
     static const char* launch_name(const lbm_handle* h, int j);
     static int launches(const lbm_handle* h);
     static int init(lbm_handle* h, const double* rho, const double* u, const double* eps);   // device pointers
-    static int moments(lbm_handle* h, double* rho, double* u, double* T, double* P);       // device pointers
+    // output fields to device-accessible pointers; the counters to *cnt_out unless null
+    static int output(lbm_handle* h, const Outputs& o, Counters* cnt_out);
     // sums over nodes [i0, i0 + n): 5 sums and 3 counters into device memory
     static int reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev);
     static size_t field_bytes(int storage);

@@ -4,7 +4,7 @@
 //   force_kernel    Phi stencil + gravity -> du = F/rho     (Sec. 3, Eq. (edm))
 //   collide_kernel  dE by finite differences, BGK + EDM for N, BGK + g dE/E +
 //                   pseudoforce for g, push streaming with walls (Eq. (lbe), (gk))
-// plus initialisation, output moments and the conservation reductions.
+// plus initialisation and the conservation reductions.
 //
 // Populations: Q arrays of nn node pairs (N_k, g_k), nn = nx*ny*nz, x fastest
 // (lattice.cuh); checkpoints use 2Q set-major planes.  Fields: planes of nn
@@ -258,24 +258,6 @@ __global__ void __launch_bounds__(256) init_kernel(S* __restrict__ pop, const do
         Store<S, R>::store2(pop, pair_index(k, nn, i), rho * e0, E * e0, wk * p.rho_ref, wk * p.E_ref,
                             pair_word(nbits, k));
     }
-}
-
-// Output fields after fields_kernel + force_kernel: rho, u* = u + du/2
-// (Eq. (ustar)), T and P (EOS).
-template <int Q, typename R>
-__global__ void __launch_bounds__(256) output_kernel(const R* __restrict__ fld, KParams<R> p, double* rho,
-                                                     double* u, double* T, double* P) {
-    constexpr int D = Vel<Q>::D;
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.nn) return;
-    const long long nn = p.nn;
-    const R r = fld[F_RHO * nn + i], t = fld[F_T * nn + i];
-    if (rho) rho[i] = (double)r;
-    if (T) T[i] = (double)t;
-    if (P) P[i] = (double)eos_pressure(p, r, t);
-    if (u)
-        for (int a = 0; a < D; ++a)
-            u[a * nn + i] = (double)(fld[(F_UX + a) * nn + i] + fld[(F_DUX + a) * nn + i] / R(2));
 }
 
 // ---------------------------------------------------------------------------

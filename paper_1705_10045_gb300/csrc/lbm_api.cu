@@ -139,16 +139,6 @@ int be_step(lbm_handle* h, int n) {
 int be_init(lbm_handle* h, const double* r, const double* u, const double* e) {
     return h->Q == 9 ? lbm::Backend<9>::init(h, r, u, e) : lbm::Backend<19>::init(h, r, u, e);
 }
-int be_moments(lbm_handle* h, double* r, double* u, double* T, double* P) {
-    return h->Q == 9 ? lbm::Backend<9>::moments(h, r, u, T, P) : lbm::Backend<19>::moments(h, r, u, T, P);
-}
-
-// FP64 -> FP32, round to nearest (the FP32 twin of the moments)
-__global__ void narrow_kernel(const double* __restrict__ src, float* __restrict__ dst, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dst[i] = (float)src[i];
-}
-
 // Report what the device counters say since the last report.
 int latch(lbm_handle* h, unsigned long long bad, unsigned long long timeouts) {
     if (timeouts) {
@@ -174,6 +164,60 @@ int sync_and_latch(lbm_handle* h) {
     rc = cuda_error(cudaStreamSynchronize(h->stream), "stream synchronize");
     if (rc) return rc;
     return latch(h, c.bad, c.timeouts);
+}
+
+int be_output(lbm_handle* h, const lbm::Outputs& o, lbm::Counters* cnt_out) {
+    return h->Q == 9 ? lbm::Backend<9>::output(h, o, cnt_out) : lbm::Backend<19>::output(h, o, cnt_out);
+}
+
+// Host outputs of at most this many bytes are written by the kernels straight
+// into a pinned buffer, with the counters, and copied from there by the host:
+// every copy from the device to pageable memory takes about 8 us, whatever its
+// size (a row of 128 nodes: four fields and the counters 80 us -> 35 us).
+constexpr size_t kBounceBytes = 128 << 10;
+
+// The output fields of the current state.
+int output_fields(lbm_handle* h, const lbm::Outputs& o, int mem) {
+    DeviceGuard dg(h->p.device);
+    int rc;
+    if (mem == LBM_MEM_DEVICE) {
+        if ((rc = be_output(h, o, nullptr))) return rc;
+        return sync_and_latch(h);
+    }
+    const size_t elem = o.single ? sizeof(float) : sizeof(double), plane = elem * (size_t)h->nn;
+    struct Field {
+        void* dst;
+        size_t bytes;
+        unsigned char* dev;
+    } f[4] = {{o.rho, plane, nullptr}, {o.u, plane * h->D, nullptr}, {o.T, plane, nullptr}, {o.P, plane, nullptr}};
+    const size_t total = plane * (size_t)(h->D + 3), counters = (sizeof(lbm::Counters) + 63) & ~(size_t)63;
+    const bool small = total <= kBounceBytes;
+    if (small && !h->bounce) {   // room for doubles, should the next call ask for them
+        const size_t most = std::min(kBounceBytes, sizeof(double) * (size_t)(h->D + 3) * (size_t)h->nn);
+        if ((rc = cuda_error(cudaMallocHost(&h->bounce, counters + most), "output buffer allocation"))) return rc;
+    }
+    // FP32 outputs of larger domains stage in the idle population buffer (at
+    // least (d + 3) floats per node in every storage format)
+    if (!small && !o.single && (rc = ensure_staging(h))) return rc;
+    unsigned char* at = small ? (unsigned char*)h->bounce + counters
+                              : (unsigned char*)(o.single ? h->pop[h->cur ^ 1] : (void*)h->staging);
+    for (Field& x : f) {
+        if (x.dst) x.dev = at;
+        at += x.bytes;
+    }
+    auto* cnt = small ? (lbm::Counters*)h->bounce : nullptr;
+    if ((rc = be_output(h, {f[0].dev, f[1].dev, f[2].dev, f[3].dev, o.single}, cnt))) return rc;
+    if (small) {
+        if ((rc = cuda_error(cudaStreamSynchronize(h->stream), "stream synchronize"))) return rc;
+        for (const Field& x : f)
+            if (x.dst) std::memcpy(x.dst, x.dev, x.bytes);
+        return latch(h, cnt->bad, cnt->timeouts);
+    }
+    for (const Field& x : f)
+        if (x.dst && (rc = cuda_error(cudaMemcpyAsync(x.dst, x.dev, x.bytes, cudaMemcpyDeviceToHost, h->stream),
+                                      "moments copy")))
+            return rc;
+    return sync_and_latch(h);
 }
 
 }  // namespace
@@ -428,28 +472,7 @@ int lbm_moments(lbm_handle* h, double* rho, double* u, double* T, double* P, int
         set_error("lbm_moments: bad mem flag");
         return LBM_ERR_INVALID_ARG;
     }
-    DeviceGuard dg(h->p.device);
-    int rc;
-    if (mem == LBM_MEM_DEVICE) {
-        if ((rc = be_moments(h, rho, u, T, P))) return rc;
-        return sync_and_latch(h);
-    }
-    if ((rc = ensure_staging(h))) return rc;
-    const long long nn = h->nn;
-    double* s = h->staging;
-    double *dr = rho ? s : nullptr, *du = u ? s + nn : nullptr, *dT = T ? s + (1 + h->D) * nn : nullptr,
-           *dP = P ? s + (2 + h->D) * nn : nullptr;
-    if ((rc = be_moments(h, dr, du, dT, dP))) return rc;
-    const size_t plane = sizeof(double) * (size_t)nn;
-    if (rho && (rc = cuda_error(cudaMemcpyAsync(rho, dr, plane, cudaMemcpyDeviceToHost, h->stream), "moments copy")))
-        return rc;
-    if (u && (rc = cuda_error(cudaMemcpyAsync(u, du, plane * h->D, cudaMemcpyDeviceToHost, h->stream), "moments copy")))
-        return rc;
-    if (T && (rc = cuda_error(cudaMemcpyAsync(T, dT, plane, cudaMemcpyDeviceToHost, h->stream), "moments copy")))
-        return rc;
-    if (P && (rc = cuda_error(cudaMemcpyAsync(P, dP, plane, cudaMemcpyDeviceToHost, h->stream), "moments copy")))
-        return rc;
-    return sync_and_latch(h);
+    return output_fields(h, {rho, u, T, P, false}, mem);
 }
 
 int lbm_moments_f(lbm_handle* h, float* rho, float* u, float* T, float* P, int mem) {
@@ -461,36 +484,7 @@ int lbm_moments_f(lbm_handle* h, float* rho, float* u, float* T, float* P, int m
         set_error("lbm_moments_f: bad mem flag");
         return LBM_ERR_INVALID_ARG;
     }
-    DeviceGuard dg(h->p.device);
-    int rc;
-    if ((rc = ensure_staging(h))) return rc;
-    const long long nn = h->nn;
-    double* s = h->staging;
-    double *dr = rho ? s : nullptr, *du = u ? s + nn : nullptr, *dT = T ? s + (1 + h->D) * nn : nullptr,
-           *dP = P ? s + (2 + h->D) * nn : nullptr;
-    if ((rc = be_moments(h, dr, du, dT, dP))) return rc;
-    // the floats: straight into device outputs, or into the idle population
-    // buffer (at least (d + 3) floats per node in every storage format)
-    float* idle = static_cast<float*>(h->pop[h->cur ^ 1]);
-    struct Field {
-        const double* src;
-        float* dst;
-        long long n;
-    } fields[4] = {{dr, rho, nn}, {du, u, h->D * nn}, {dT, T, nn}, {dP, P, nn}};
-    long long off = 0;
-    for (const Field& f : fields) {
-        if (!f.dst) continue;
-        float* d = mem == LBM_MEM_DEVICE ? f.dst : idle + off;
-        const unsigned blocks = (unsigned)std::min<long long>((f.n + 255) / 256, 4096);
-        narrow_kernel<<<blocks, 256, 0, h->stream>>>(f.src, d, f.n);
-        if ((rc = cuda_error(cudaGetLastError(), "moments narrowing launch"))) return rc;
-        if (mem == LBM_MEM_HOST &&
-            (rc = cuda_error(cudaMemcpyAsync(f.dst, d, sizeof(float) * (size_t)f.n, cudaMemcpyDeviceToHost, h->stream),
-                             "moments copy")))
-            return rc;
-        off += f.n;
-    }
-    return sync_and_latch(h);
+    return output_fields(h, {rho, u, T, P, true}, mem);
 }
 
 int lbm_diagnostics(lbm_handle* h, double out[8]) {
@@ -634,6 +628,7 @@ void lbm_destroy(lbm_handle* h) {
     cudaFree(h->partials);
     cudaFree(h->staging);
     cudaFree(h->coex);
+    cudaFreeHost(h->bounce);
     delete h;
 }
 

@@ -26,6 +26,40 @@ template <> struct MVel<19> {
     __host__ __device__ static constexpr int m(int k) { return Vel<19>::cz(k); }
 };
 
+// Offsets of the neighbours of node n along its lattice axes.  lo / hi: the
+// node a stencil reads (across a wall the mirror node, the node itself);
+// wrap_lo / wrap_hi: the periodic neighbour; g: walls beside the node (bit 2a
+// the low one of axis a, bit 2a + 1 the high one).
+template <int Q, typename R> struct NodeSteps {
+    int lo[3], hi[3], wrap_lo[3], wrap_hi[3], g;
+    __device__ __forceinline__ NodeSteps(const KParams<R>& p, int n) {
+        constexpr int D = Vel<Q>::D;
+        int c[3];
+        node_xyz(n, p.nx, p.ny, c[0], c[1], c[2]);
+        const int len[3] = {p.nx, p.ny, p.nz}, stride[3] = {1, p.nx, p.nx * p.ny};
+        g = 0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const bool wall = a == D - 1 ? p.wall : (a == 0 ? p.wall_x : p.wall_y);
+            wrap_lo[a] = c[a] == 0 ? (len[a] - 1) * stride[a] : -stride[a];
+            wrap_hi[a] = c[a] == len[a] - 1 ? -(len[a] - 1) * stride[a] : stride[a];
+            const bool l = wall && c[a] == 0, h = wall && c[a] == len[a] - 1;
+            lo[a] = l ? 0 : wrap_lo[a];
+            hi[a] = h ? 0 : wrap_hi[a];
+            g |= (l ? 1 : 0) << (2 * a) | (h ? 2 : 0) << (2 * a);
+        }
+    }
+    // the node at n + c_k as a stencil reads it
+    __device__ __forceinline__ int at(int n, int k) const {
+        using V = Vel<Q>;
+        const int c[3] = {V::cx(k), V::cy(k), V::cz(k)};
+#pragma unroll
+        for (int a = 0; a < V::D; ++a)
+            if (c[a] != 0) n += c[a] > 0 ? hi[a] : lo[a];
+        return n;
+    }
+};
+
 // Two values moved through the same operation: the N and g of a direction.
 // FP32 uses the packed instructions (one issue slot for both, each half
 // rounded as the scalar instruction rounds it).

@@ -43,6 +43,7 @@ template <int Q, typename S, typename R> struct Phase {
     using M = MVel<Q>;
     using Math = NodeMath<Q, S, R>;
     static constexpr int D = V::D;
+    using Steps = NodeSteps<Q, R>;
 
     // node of this thread, or -1
     __device__ static __forceinline__ int node(const PhaseGeom& G) {
@@ -50,29 +51,6 @@ template <int Q, typename S, typename R> struct Phase {
         if (t >= (unsigned)G.count * (unsigned)G.plane_n) return -1;
         const unsigned all = (unsigned)G.nm * (unsigned)G.plane_n, n = (unsigned)G.first * (unsigned)G.plane_n + t;
         return (int)(n >= all ? n - all : n);
-    }
-    // offsets of the neighbours of a node along its axes; across a wall the
-    // mirror node is the node itself (g: bit 2a low, bit 2a + 1 high)
-    struct Steps {
-        int lo[3], hi[3], wrap_lo[3], wrap_hi[3], g;
-    };
-    __device__ static __forceinline__ Steps steps(const KParams<R>& p, int n) {
-        int c[3];
-        node_xyz(n, p.nx, p.ny, c[0], c[1], c[2]);
-        const int len[3] = {p.nx, p.ny, p.nz}, stride[3] = {1, p.nx, p.nx * p.ny};
-        Steps s;
-        s.g = 0;
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const bool wall = a == D - 1 ? p.wall : (a == 0 ? p.wall_x : p.wall_y);
-            s.wrap_lo[a] = c[a] == 0 ? (len[a] - 1) * stride[a] : -stride[a];
-            s.wrap_hi[a] = c[a] == len[a] - 1 ? -(len[a] - 1) * stride[a] : stride[a];
-            const bool l = wall && c[a] == 0, h = wall && c[a] == len[a] - 1;
-            s.lo[a] = l ? 0 : s.wrap_lo[a];
-            s.hi[a] = h ? 0 : s.wrap_hi[a];
-            s.g |= (l ? 1 : 0) << (2 * a) | (h ? 2 : 0) << (2 * a);
-        }
-        return s;
     }
     // lattice axis of march axis 0 (a), 1 (b), 2 (m)
     __device__ static constexpr int axis(int march) { return Q == 9 && march == 2 ? 1 : march; }
@@ -120,7 +98,7 @@ __global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, c
     const int n = Ph::node(G);
     if (n < 0) return;
     const size_t nn = (size_t)p.nn;
-    const typename Ph::Steps s = Ph::steps(p, n);
+    const typename Ph::Steps s(p, n);
     const R* phi = fld + F_PHI * nn;
     R du[3];
     NodeMath<Q, S, R>::force(p, [&](int a, int b, int m) {
@@ -147,7 +125,7 @@ __global__ void __launch_bounds__(128) phase_collide_kernel(const S* __restrict_
     const int n = Ph::node(G);
     if (n < 0) return;
     const size_t nn = (size_t)p.nn;
-    const typename Ph::Steps s = Ph::steps(p, n);
+    const typename Ph::Steps s(p, n);
     Pop<S> f[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) f[k] = load_pop<false>(src + 2 * ((size_t)k * nn), (size_t)n);
