@@ -77,18 +77,17 @@ template <typename R> struct FusedTile<9, R> { static constexpr int TX = 128, TY
 template <> struct FusedTile<19, float> { static constexpr int TX = 32, TY = 8, NP = 128; static constexpr bool SPLIT = true; };
 template <> struct FusedTile<19, double> { static constexpr int TX = 32, TY = 8, NP = 256; static constexpr bool SPLIT = true; };
 
-// CTA shapes a batch may run with (TX x TY consumers + NP producers); the
-// autotuner times each on the batch and keeps the fastest.
-// MB: CTAs per SM the batch kernel is compiled for (its register cap).
-// SPLIT: as for the single-domain step (D3Q19: consumers form their own
-// nodes' moments).
-template <int Q, typename R, int V> struct BatchShape;
-template <typename R> struct BatchShape<9, R, 0> { static constexpr int TX = 128, TY = 1, NP = 160, MB = 3; static constexpr bool SPLIT = false; };
-template <typename R> struct BatchShape<9, R, 1> { static constexpr int TX = 32, TY = 1, NP = 32, MB = 16; static constexpr bool SPLIT = false; };
-template <typename R> struct BatchShape<9, R, 2> { static constexpr int TX = 64, TY = 1, NP = 64, MB = 8; static constexpr bool SPLIT = false; };
-template <typename R> struct BatchShape<19, R, 0> { static constexpr int TX = 32, TY = 8, NP = 128, MB = 2; static constexpr bool SPLIT = true; };
-template <typename R> struct BatchShape<19, R, 1> { static constexpr int TX = 32, TY = 8, NP = 160, MB = 2; static constexpr bool SPLIT = true; };
-template <typename R> struct BatchShape<19, R, 2> { static constexpr int TX = 32, TY = 4, NP = 96, MB = 3; static constexpr bool SPLIT = true; };
+// CTA shapes a batch may run with; the autotuner times each on the batch and
+// keeps the fastest.  D2Q9: W warps of a strip each.  D3Q19: TX x TY consumers
+// + NP producers of the march, its moment stage split.  MB: CTAs per SM the
+// batch kernel is compiled for (its register cap).
+template <int Q, int V> struct BatchShape;
+template <> struct BatchShape<9, 0> { static constexpr int W = 4, MB = 4; };
+template <> struct BatchShape<9, 1> { static constexpr int W = 1, MB = 16; };
+template <> struct BatchShape<9, 2> { static constexpr int W = 2, MB = 8; };
+template <> struct BatchShape<19, 0> { static constexpr int TX = 32, TY = 8, NP = 128, MB = 2; };
+template <> struct BatchShape<19, 1> { static constexpr int TX = 32, TY = 8, NP = 160, MB = 2; };
+template <> struct BatchShape<19, 2> { static constexpr int TX = 32, TY = 4, NP = 96, MB = 3; };
 
 template <int Q, typename S, typename R> struct Impl {
     static constexpr int TX = FusedTile<Q, R>::TX, TY = FusedTile<Q, R>::TY, NP = FusedTile<Q, R>::NP;
@@ -180,7 +179,7 @@ template <int Q, typename S, typename R> struct Impl {
     static StripGeom strip_geometry(const MarchGeom& G) {
         StripGeom s;
         s.na = G.na; s.nm = G.nm; s.m_lo = G.m_lo; s.m_hi = G.m_hi;
-        s.strips = (G.na + Strip<S, R, false>::kCols - 1) / Strip<S, R, false>::kCols;
+        s.strips = strip_count(G.na);
         s.chunk = strip_rows(s.strips, G.m_hi - G.m_lo, kSms);
         return s;
     }
@@ -351,12 +350,26 @@ template <int Q, typename S, typename R> struct Impl {
         return cuda_error(cudaGetLastError(), "lbm_moments launch");
     }
     // ---- batches ---------------------------------------------------------
-    // CTA shapes a batch can run with; the autotuner picks one per batch
-    template <int V> struct Shape;
-    static constexpr int kVariants = 3;
-
-    template <int BTX, int BTY, int BNP, int BMB>
-    static MarchGeom batch_geometry(const lbm_handle* h) {
+    // Planes (D2Q9: rows) per work item of the domains that step in a request.
+    // D3Q19: 64.  D2Q9: a step of a domain starts when all items of its
+    // previous step are done, so an item (its rows and four more at 1.45 us
+    // with 16 warps per SM, 2 us to hand over) should take no longer than 3/4
+    // of what one step of every domain takes (1.45 us per 16 x 152 warp rows),
+    // within 2 to 64 rows.  Measured us per step of every domain: 24 domains of
+    // 64..512 (2.9 M nodes; 29 rows) 16 rows 81.5, 32 rows 75.6, 64 rows 88.8;
+    // 6 of 64..200 (2 rows) 2 rows 8.9, 4 rows 10.5, 8 rows 13.7; 64 of 64..512 (64 rows) 32
+    // rows 157, 64 rows 153.
+    static int batch_chunk(const lbm_batch* b) {
+        if (Q == 19) return 64;
+        double rows = 0;   // warp rows of one step of every domain
+        for (size_t d = 0; d < b->doms.size(); ++d)
+            if (d < b->in_table.size() && b->in_table[d]) rows += (double)strip_count(b->doms[d]->p.nx) * b->doms[d]->p.ny;
+        const double step = rows * 1.45 / (16.0 * kSms);
+        const int c = (int)((0.75 * step - 2.0) / 1.45) - 4;
+        return c < 2 ? 2 : (c > 64 ? 64 : c);
+    }
+    template <typename B>
+    static MarchGeom batch_geometry(const lbm_handle* h, int chunk) {
         MarchGeom G;
         G.na = h->p.nx;
         G.nb = Q == 9 ? 1 : h->p.ny;
@@ -365,38 +378,70 @@ template <int Q, typename S, typename R> struct Impl {
         // the ring planes at its ends and, with the split moment stage, forms
         // the moments of its first three planes in the producers alone, so long
         // items pay; the items of the other domains of a batch fill the waves
-        // (measured: shorter items for four waves per domain gave 31 instead of
-        // 40 jobs/s on the D2Q9 batch and 2.1 instead of 2.4 served jobs/s)
-        G.chunk = G.nm < 64 ? G.nm : 64;
+        // (measured: shorter items for four waves per domain gave 2.1 instead
+        // of 2.4 served jobs/s)
+        G.chunk = G.nm < chunk ? G.nm : chunk;
         G.m_lo = 0;
         G.m_hi = G.nm;
         return G;
     }
 
-    template <int BTX, int BTY, int BNP, int BMB, bool BSP>
-    static int build_shape(lbm_batch* b) {
+    // the batch kernel of shape B: with the fault-injection hook, for domains
+    // with walls across the march, for the others
+    static constexpr int kFault = 0, kWalls = 1, kPlain = 2;
+    template <typename B> static const void* batch_kernel(int which) {
+        if constexpr (Q == 9) {
+            return which == kFault   ? (const void*)strip_batch_kernel<S, R, B::W, B::MB, true, true>
+                   : which == kWalls ? (const void*)strip_batch_kernel<S, R, B::W, B::MB, false, true>
+                                     : (const void*)strip_batch_kernel<S, R, B::W, B::MB, false, false>;
+        } else {
+            return which == kFault   ? (const void*)fused_batch_kernel<Q, S, R, B::TX, B::TY, B::NP, B::MB, true, true, true>
+                   : which == kWalls ? (const void*)fused_batch_kernel<Q, S, R, B::TX, B::TY, B::NP, B::MB, false, true, true>
+                                     : (const void*)fused_batch_kernel<Q, S, R, B::TX, B::TY, B::NP, B::MB, false, false, true>;
+        }
+    }
+    template <typename B> static constexpr int batch_threads() {
+        if constexpr (Q == 9) return 32 * B::W;
+        else return B::TX * B::TY + B::NP;
+    }
+    template <typename B> static constexpr size_t batch_smem() {
+        if constexpr (Q == 9) return B::W * Strip<S, R, true>::kRingBytes;
+        else return FusedShape<B::TX, B::TY, true>::template smem_bytes<R>();
+    }
+    static bool has_walls(const lbm_handle* h) {
+        return Q == 9 ? h->p.wall || h->p.wall_x : h->p.wall_x || h->p.wall_y;
+    }
+
+    template <typename B> static int build_shape(lbm_batch* b) {
         std::vector<BatchItem> items;
         DomainDesc<R>* descs = (DomainDesc<R>*)b->h_descs;
+        const int chunk = batch_chunk(b);
         for (size_t d = 0; d < b->doms.size(); ++d) {
             lbm_handle* h = b->doms[d];
             DomainDesc<R> dd{};
             if (h) {
                 dd.kp = make_kparams<R>(h);
-                dd.G = batch_geometry<BTX, BTY, BNP, BMB>(h);
+                dd.G = batch_geometry<B>(h, chunk);
                 dd.pop[0] = h->pop[0];
                 dd.pop[1] = h->pop[1];
                 dd.cnt = (Counters*)h->cnt;
                 dd.cur = h->cur;
                 dd.left = 0;
-                const int tx = (dd.G.na + BTX - 1) / BTX, ty = (dd.G.nb + BTY - 1) / BTY;
                 const int tz = (dd.G.nm + dd.G.chunk - 1) / dd.G.chunk;
-                dd.n_items = tx * ty * tz;
                 // only the domains that step in this request get work items: a
                 // paused domain would cost every persistent CTA a pass over them
-                if (d < b->in_table.size() && b->in_table[d])
-                    for (int z = 0; z < tz; ++z)
+                const bool in = d < b->in_table.size() && b->in_table[d];
+                if constexpr (Q == 9) {
+                    const int warps = strip_count(dd.G.na) * tz;
+                    dd.n_items = (warps + B::W - 1) / B::W;
+                    for (int w = 0; in && w < warps; w += B::W) items.push_back({(int)d, w, 0, 0});
+                } else {
+                    const int tx = (dd.G.na + B::TX - 1) / B::TX, ty = (dd.G.nb + B::TY - 1) / B::TY;
+                    dd.n_items = tx * ty * tz;
+                    for (int z = 0; in && z < tz; ++z)
                         for (int y = 0; y < ty; ++y)
-                            for (int x = 0; x < tx; ++x) items.push_back({(int)d, x * BTX, y * BTY, z * dd.G.chunk});
+                            for (int x = 0; x < tx; ++x) items.push_back({(int)d, x * B::TX, y * B::TY, z * dd.G.chunk});
+                }
             }
             descs[d] = dd;
         }
@@ -413,19 +458,17 @@ template <int Q, typename S, typename R> struct Impl {
                                                     cudaMemcpyHostToDevice, b->stream), "batch table copy"))
                 return rc;
         // one persistent CTA per resident slot: occupancy times the SM count
-        const size_t smem = FusedShape<BTX, BTY, BSP>::template smem_bytes<R>();
+        constexpr size_t smem = batch_smem<B>();
         b->xw = false;
-        for (auto* h : b->doms) b->xw = b->xw || (h && (h->p.wall_x || (Q == 19 && h->p.wall_y)));
-        const void* kerns[3] = {(const void*)fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, true, true, BSP>,
-                                (const void*)fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, false, true, BSP>,
-                                (const void*)fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, false, false, BSP>};
-        for (const void* kern : kerns)
-            if (int rc = cuda_error(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        for (auto* h : b->doms) b->xw = b->xw || (h && has_walls(h));
+        for (int which : {kFault, kWalls, kPlain})
+            if (int rc = cuda_error(cudaFuncSetAttribute(batch_kernel<B>(which),
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                                     "batch kernel attribute"))
                 return rc;
         int per_sm = 0, sms = 0;
-        if (int rc = cuda_error(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kerns[b->xw ? 1 : 2],
-                                                                              BTX * BTY + BNP, smem),
+        if (int rc = cuda_error(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                    &per_sm, batch_kernel<B>(b->xw ? kWalls : kPlain), batch_threads<B>(), smem),
                                 "batch occupancy"))
             return rc;
         if (int rc = cuda_error(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->common.device),
@@ -436,23 +479,12 @@ template <int Q, typename S, typename R> struct Impl {
     }
 
     // the persistent launch of a request (steps and scheduling state already in device memory)
-    template <int BTX, int BTY, int BNP, int BMB, bool BSP>
-    static void launch_shape(lbm_batch* b) {
-        const size_t smem = FusedShape<BTX, BTY, BSP>::template smem_bytes<R>();
-        const int n_doms = (int)b->doms.size();
+    template <typename B> static void launch_shape(lbm_batch* b) {
+        int n_items = b->n_items, n_doms = (int)b->doms.size(), fault = b->fault_item >= 0 ? b->fault_item : -1;
         const int grid = std::max(1, b->grid);   // CTAs beyond the work of a request leave at once
-        const auto* items = (const BatchItem*)b->d_items;
-        const auto* descs = (const DomainDesc<R>*)b->d_descs;
-        auto* sched = (BatchSched*)b->d_sched;
-        if (b->fault_item >= 0)
-            fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, true, true, BSP><<<grid, BTX * BTY + BNP, smem, b->stream>>>(
-                items, descs, b->n_items, sched, n_doms, b->fault_item);
-        else if (b->xw)
-            fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, false, true, BSP><<<grid, BTX * BTY + BNP, smem, b->stream>>>(
-                items, descs, b->n_items, sched, n_doms, -1);
-        else
-            fused_batch_kernel<Q, S, R, BTX, BTY, BNP, BMB, false, false, BSP><<<grid, BTX * BTY + BNP, smem, b->stream>>>(
-                items, descs, b->n_items, sched, n_doms, -1);
+        void* args[] = {&b->d_items, &b->d_descs, &n_items, &b->d_sched, &n_doms, &fault};
+        cudaLaunchKernel(batch_kernel<B>(fault >= 0 ? kFault : (b->xw ? kWalls : kPlain)), dim3(grid),
+                         dim3(batch_threads<B>()), args, batch_smem<B>(), b->stream);
     }
 
     static int batch_build(lbm_batch* b);
@@ -471,9 +503,9 @@ template <int Q, typename S, typename R> struct Impl {
 
 template <int Q, typename S, typename R> int Impl<Q, S, R>::batch_build(lbm_batch* b) {
     switch (b->variant) {
-        case 0: return build_shape<BatchShape<Q, R, 0>::TX, BatchShape<Q, R, 0>::TY, BatchShape<Q, R, 0>::NP, BatchShape<Q, R, 0>::MB, BatchShape<Q, R, 0>::SPLIT>(b);
-        case 1: return build_shape<BatchShape<Q, R, 1>::TX, BatchShape<Q, R, 1>::TY, BatchShape<Q, R, 1>::NP, BatchShape<Q, R, 1>::MB, BatchShape<Q, R, 1>::SPLIT>(b);
-        default: return build_shape<BatchShape<Q, R, 2>::TX, BatchShape<Q, R, 2>::TY, BatchShape<Q, R, 2>::NP, BatchShape<Q, R, 2>::MB, BatchShape<Q, R, 2>::SPLIT>(b);
+        case 0: return build_shape<BatchShape<Q, 0>>(b);
+        case 1: return build_shape<BatchShape<Q, 1>>(b);
+        default: return build_shape<BatchShape<Q, 2>>(b);
     }
 }
 
@@ -485,9 +517,9 @@ template <int Q, typename S, typename R> int Impl<Q, S, R>::batch_launch(lbm_bat
         if (int rc = cuda_error(cudaMemsetAsync((char*)b->d_sched + sizeof(int), 0, clear, b->stream), "batch clear"))
             return rc;
         switch (b->variant) {
-            case 0: launch_shape<BatchShape<Q, R, 0>::TX, BatchShape<Q, R, 0>::TY, BatchShape<Q, R, 0>::NP, BatchShape<Q, R, 0>::MB, BatchShape<Q, R, 0>::SPLIT>(b); break;
-            case 1: launch_shape<BatchShape<Q, R, 1>::TX, BatchShape<Q, R, 1>::TY, BatchShape<Q, R, 1>::NP, BatchShape<Q, R, 1>::MB, BatchShape<Q, R, 1>::SPLIT>(b); break;
-            default: launch_shape<BatchShape<Q, R, 2>::TX, BatchShape<Q, R, 2>::TY, BatchShape<Q, R, 2>::NP, BatchShape<Q, R, 2>::MB, BatchShape<Q, R, 2>::SPLIT>(b); break;
+            case 0: launch_shape<BatchShape<Q, 0>>(b); break;
+            case 1: launch_shape<BatchShape<Q, 1>>(b); break;
+            default: launch_shape<BatchShape<Q, 2>>(b); break;
         }
     }
     if (advance && !b->doms.empty()) {
@@ -544,7 +576,7 @@ template <int Q> int Backend<Q>::reduce(lbm_handle* h, long long i0, long long n
     }
 template <int Q> int Backend<Q>::batch_variants() { return 3; }
 template <int Q> const char* Backend<Q>::batch_variant_name(int v) {
-    static const char* n9[] = {"128x1+160", "32x1+32", "64x1+64"};
+    static const char* n9[] = {"4 strips", "1 strip", "2 strips"};
     static const char* n19[] = {"32x8+128", "32x8+160", "32x4+96"};
     if (v < 0 || v > 2) return "";
     return Q == 9 ? n9[v] : n19[v];

@@ -42,6 +42,7 @@
 #pragma once
 
 #include "node.cuh"
+#include "strip.cuh"
 
 namespace lbm {
 
@@ -561,15 +562,13 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     return v;
 }
 
-// FAULT: the item fault_item of step 0 does not report its completion
-// (tests of the bounded waits only).  XW: some domain has walls on the
-// tile-plane axes.  SPLIT: the consumers form their own nodes' moments.
-template <int Q, typename S, typename R, int TX, int TY, int NP, int MB, bool FAULT, bool XW, bool SPLIT>
-__global__ void __launch_bounds__(TX* TY + NP, MB) fused_batch_kernel(const BatchItem* __restrict__ items,
-                                                                  const DomainDesc<R>* __restrict__ doms,
-                                                                  int n_items, BatchSched* sched, int n_doms,
-                                                                  int fault_item) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+// The scheduling loop of a persistent CTA.  work(item, domain, kp, s): step s
+// of a work item, by every thread of the CTA; kp: the CTA's copy of the
+// domain's parameters.  FAULT: the item fault_item of step 0 does not report
+// its completion (tests of the bounded waits only).
+template <bool FAULT, typename R, typename W>
+__device__ __forceinline__ void batch_loop(const BatchItem* __restrict__ items, const DomainDesc<R>* __restrict__ doms,
+                                           int n_items, BatchSched* sched, int n_doms, int fault_item, const W& work) {
     __shared__ KParams<R> kp;   // the current item's domain parameters
     __shared__ int w_sh, go_sh;
     int kp_domain = -1;         // domain whose parameters kp holds (thread 0)
@@ -610,13 +609,7 @@ __global__ void __launch_bounds__(TX* TY + NP, MB) fused_batch_kernel(const Batc
             go_sh = go;
         }
         __syncthreads();
-        if (active && go_sh) {
-            const int in = (d->cur + s) & 1;
-            const MarchGeom G = d->G;
-            fused_tile<Q, S, R, TX, TY, NP, false, true, XW, SPLIT>((const S*)d->pop[in], (S*)d->pop[in ^ 1], &kp, G,
-                                                         kp.step + (unsigned)s, it.a0, it.b0, it.zb, d->cnt,
-                                                         smem_raw);
-        }
+        if (active && go_sh) work(it, d, kp, s);
         __syncthreads();
         if (active && threadIdx.x == 0) {
             bool report = true;
@@ -627,6 +620,49 @@ __global__ void __launch_bounds__(TX* TY + NP, MB) fused_batch_kernel(const Batc
             }
         }
     }
+}
+
+// Items are tiles and chunks of planes of the march.  XW: some domain has
+// walls on the tile-plane axes.  SPLIT: the consumers form their own nodes'
+// moments.
+template <int Q, typename S, typename R, int TX, int TY, int NP, int MB, bool FAULT, bool XW, bool SPLIT>
+__global__ void __launch_bounds__(TX* TY + NP, MB) fused_batch_kernel(const BatchItem* __restrict__ items,
+                                                                  const DomainDesc<R>* __restrict__ doms,
+                                                                  int n_items, BatchSched* sched, int n_doms,
+                                                                  int fault_item) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    batch_loop<FAULT, R>(items, doms, n_items, sched, n_doms, fault_item,
+                         [&](const BatchItem& it, const DomainDesc<R>* d, const KParams<R>& kp, int s) {
+        const int in = (d->cur + s) & 1;
+        const MarchGeom G = d->G;
+        fused_tile<Q, S, R, TX, TY, NP, false, true, XW, SPLIT>((const S*)d->pop[in], (S*)d->pop[in ^ 1], &kp, G,
+                                                     kp.step + (unsigned)s, it.a0, it.b0, it.zb, d->cnt, smem_raw);
+    });
+}
+
+// D2Q9: items are groups of W strips of a domain (strip.cuh), numbered strip
+// first, then chunk of rows; it.a0 is the first of the group.  Strips copy
+// their rows with cp.async, which reads what the domain's other CTAs wrote in
+// the previous step: every thread issues it after the acquire that the CTA's
+// first thread made and the barrier behind it.
+template <typename S, typename R, int W, int MB, bool FAULT, bool WALL>
+__global__ void __launch_bounds__(32 * W, MB) strip_batch_kernel(const BatchItem* __restrict__ items,
+                                                                 const DomainDesc<R>* __restrict__ doms, int n_items,
+                                                                 BatchSched* sched, int n_doms, int fault_item) {
+    using St = Strip<S, R, WALL>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5;
+    batch_loop<FAULT, R>(items, doms, n_items, sched, n_doms, fault_item,
+                         [&](const BatchItem& it, const DomainDesc<R>* d, const KParams<R>& kp, int s) {
+        const MarchGeom G = d->G;
+        const int strips = strip_count(G.na), w = it.a0 + warp, zb = (w / strips) * G.chunk;
+        if (zb >= G.nm) return;
+        const int in = (d->cur + s) & 1;
+        St st((const S*)d->pop[in], (S*)d->pop[in ^ 1], kp, d->cnt, G.na, G.nm, zb, min(zb + G.chunk, G.nm),
+              kp.step + (unsigned)s, (w % strips) * St::kCols,
+              reinterpret_cast<Pop<S>*>(smem_raw + warp * St::kRingBytes));
+        st.run();
+    });
 }
 
 // descriptor bookkeeping after a request of n steps: every domain took

@@ -13,6 +13,7 @@ struct lbm_handle {
     int Q = 0, D = 0;
     long long nn = 0;
     size_t elem = 0;            // bytes per stored population value
+    void* slab = nullptr;       // the allocation that holds pop, fld, cnt and partials
     void* pop[2] = {nullptr, nullptr};   // ping-pong population buffers, 2Q planes each
     int cur = 0;                // buffer holding the current state
     void* fld = nullptr;        // field planes (arithmetic type)
@@ -79,6 +80,12 @@ struct TraceRange {
 // error reporting shared by the translation units
 void set_error(const std::string& msg);
 int cuda_error(cudaError_t e, const char* where);
+// Offsets of a handle's buffers in its allocation (the first population buffer
+// at 0; every buffer 256-byte aligned).
+struct HandleLayout {
+    size_t pop1 = 0, fld = 0, cnt = 0, partials = 0, bytes = 0;
+    explicit HandleLayout(const lbm_params& p);
+};
 // lbm_create; phases: also allocate the field planes of a step in three phases,
 // for domains that step so (without them, or when there is no memory left for
 // them, those take the fused march, as the domains of a batch do)

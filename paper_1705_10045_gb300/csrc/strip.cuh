@@ -46,9 +46,12 @@ template <typename S> __device__ __forceinline__ void copy_async(Pop<S>* to, con
 
 // WALL: the domain has walls on x or y (the other instance is periodic and
 // carries no trace of them).
+constexpr int kStripCols = 28;   // columns a warp collides
+__host__ __device__ inline int strip_count(int na) { return (na + kStripCols - 1) / kStripCols; }
+
 template <typename S, typename R, bool WALL> struct Strip {
     static constexpr int Q = 9;
-    static constexpr int kCols = 28;   // columns a warp collides
+    static constexpr int kCols = kStripCols;
     // rows a warp holds: the two loaded ahead of the moments, the row the
     // moments take and the one between it and the collision's (whose slot the
     // next load reuses)
