@@ -351,35 +351,51 @@ template <int Q, typename S, typename R> struct Impl {
     }
     // ---- batches ---------------------------------------------------------
     // Planes (D2Q9: rows) per work item of the domains that step in a request.
-    // D3Q19: 64.  D2Q9: a step of a domain starts when all items of its
-    // previous step are done, so an item (its rows and four more at 1.45 us
-    // with 16 warps per SM, 2 us to hand over) should take no longer than 3/4
-    // of what one step of every domain takes (1.45 us per 16 x 152 warp rows),
-    // within 2 to 64 rows.  Measured us per step of every domain: 24 domains of
-    // 64..512 (2.9 M nodes; 29 rows) 16 rows 81.5, 32 rows 75.6, 64 rows 88.8;
-    // 6 of 64..200 (2 rows) 2 rows 8.9, 4 rows 10.5, 8 rows 13.7; 64 of 64..512 (64 rows) 32
-    // rows 157, 64 rows 153.
+    // D2Q9: a step of a domain starts when all items of its previous step are
+    // done, so an item (its rows and four more at 1.45 us with 16 warps per SM,
+    // 2 us to hand over) should take no longer than 3/4 of what one step of
+    // every domain takes (1.45 us per 16 x 152 warp rows), within 2 to 64 rows.
+    // Measured us per step of every domain: 24 domains of 64..512 (2.9 M nodes;
+    // 29 rows) 16 rows 81.5, 32 rows 75.6, 64 rows 88.8; 6 of 64..200 (2 rows) 2
+    // rows 8.9, 4 rows 10.5, 8 rows 13.7; 64 of 64..512 (64 rows) 32 rows 157, 64
+    // rows 153.
+    // D3Q19: the chunk of up to 64 planes with the smallest modelled time of one
+    // step of every domain, (planes + 4.5) times the time of a plane (as in
+    // march_chunk) times the waves of CTAs; long items repeat fewer ring planes,
+    // and only few or small domains need shorter ones to fill the chip.
+    // Measured FP32, 64 planes -> this: 126^3 + 80^3 315 -> 215 us, four of 64^3
+    // 259 -> 83, 33^3 + 46^3 + 63^3 243 -> 49, eight of 33..126 480 (64 planes).
     static int batch_chunk(const lbm_batch* b) {
-        if (Q == 19) return 64;
-        double rows = 0;   // warp rows of one step of every domain
+        std::vector<MarchGeom> in;
         for (size_t d = 0; d < b->doms.size(); ++d)
-            if (d < b->in_table.size() && b->in_table[d]) rows += (double)strip_count(b->doms[d]->p.nx) * b->doms[d]->p.ny;
-        const double step = rows * 1.45 / (16.0 * kSms);
-        const int c = (int)((0.75 * step - 2.0) / 1.45) - 4;
-        return c < 2 ? 2 : (c > 64 ? 64 : c);
+            if (d < b->in_table.size() && b->in_table[d]) in.push_back(batch_geometry(b->doms[d], 64));
+        if (Q == 9) {
+            double rows = 0;   // warp rows of one step of every domain
+            for (const MarchGeom& G : in) rows += (double)strip_count(G.na) * G.nm;
+            const double step = rows * 1.45 / (16.0 * kSms);
+            const int c = (int)((0.75 * step - 2.0) / 1.45) - 4;
+            return c < 2 ? 2 : (c > 64 ? 64 : c);
+        }
+        int best = 64;
+        double best_t = 1e30;
+        for (int c = 2; c <= 64; ++c) {
+            long long items = 0;
+            for (const MarchGeom& G : in)
+                items += (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY) * ((G.nm + c - 1) / c);
+            const double t = (c + 4.5) * (items > kSms ? kPlane2 : kPlane1) *
+                             std::max(1.0, (double)items / (2.0 * kSms));
+            if (t <= best_t) {
+                best_t = t;
+                best = c;
+            }
+        }
+        return best;
     }
-    template <typename B>
     static MarchGeom batch_geometry(const lbm_handle* h, int chunk) {
         MarchGeom G;
         G.na = h->p.nx;
         G.nb = Q == 9 ? 1 : h->p.ny;
         G.nm = Q == 9 ? h->p.ny : h->p.nz;
-        // planes per work item: 64 (or the whole axis).  Every item recomputes
-        // the ring planes at its ends and, with the split moment stage, forms
-        // the moments of its first three planes in the producers alone, so long
-        // items pay; the items of the other domains of a batch fill the waves
-        // (measured: shorter items for four waves per domain gave 2.1 instead
-        // of 2.4 served jobs/s)
         G.chunk = G.nm < chunk ? G.nm : chunk;
         G.m_lo = 0;
         G.m_hi = G.nm;
@@ -421,7 +437,7 @@ template <int Q, typename S, typename R> struct Impl {
             DomainDesc<R> dd{};
             if (h) {
                 dd.kp = make_kparams<R>(h);
-                dd.G = batch_geometry<B>(h, chunk);
+                dd.G = batch_geometry(h, chunk);
                 dd.pop[0] = h->pop[0];
                 dd.pop[1] = h->pop[1];
                 dd.cnt = (Counters*)h->cnt;

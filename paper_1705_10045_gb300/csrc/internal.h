@@ -59,10 +59,11 @@ struct lbm_batch {
     int* h_steps = nullptr;             // pinned staging of the request's step count
     int sched_steps = 0;                // step count of the current request (host copy)
     int grid = 0;                       // persistent CTAs of the current shape
-    bool xw = false;                    // some domain has walls on the tile-plane axes
+    bool xw = false;                    // some domain has walls that the kernel has to know of
     int fault_item = -1;                // lbm_batch_test_drop_item hook: item of step 0, -1 = off
     cudaGraphExec_t graph = nullptr;    // clear + persistent launch + descriptor advance
     int graph_items = -1, graph_variant = -1, graph_doms = -1, graph_fault = -2;
+    bool graph_xw = false;
 };
 
 namespace lbm {
@@ -88,8 +89,9 @@ struct HandleLayout {
 };
 // lbm_create; phases: also allocate the field planes of a step in three phases,
 // for domains that step so (without them, or when there is no memory left for
-// them, those take the fused march, as the domains of a batch do)
+// them, those take the fused march, as the domains of a batch do together)
 int create_handle(const lbm_params* p, lbm_handle** out, bool phases);
+void ensure_phases(lbm_handle* h);   // those field planes, if the domain steps so and there is memory
 int ensure_staging(lbm_handle* h);   // the handle's host-transfer buffer, allocated on first use
 // Conservation sums of nodes [i0, i0 + n) through `partials` (block partials,
 // then 8 results): out[0..4] the sums, out[5] clamped and out[6] bad nodes.

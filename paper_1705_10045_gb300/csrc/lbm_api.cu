@@ -53,6 +53,15 @@ int ensure_staging(lbm_handle* h) {
                       "staging allocation");
 }
 
+void ensure_phases(lbm_handle* h) {
+    if (h->ext || h->p.step_kernel != LBM_STEP_FUSED) return;
+    const size_t bytes = h->Q == 9 ? Backend<9>::phase_bytes(&h->p) : Backend<19>::phase_bytes(&h->p);
+    if (bytes && cudaMalloc(&h->ext, bytes) != cudaSuccess) {
+        h->ext = nullptr;
+        (void)cudaGetLastError();   // a refused allocation is not an error of the handle
+    }
+}
+
 }  // namespace lbm
 
 using lbm::cuda_error;
@@ -363,11 +372,7 @@ int lbm::create_handle(const lbm_params* p, lbm_handle** out, bool phases) {
         lbm_destroy(h);
         return rc;
     }
-    const size_t extb = h->Q == 9 ? lbm::Backend<9>::phase_bytes(p) : lbm::Backend<19>::phase_bytes(p);
-    if (phases && extb && p->step_kernel == LBM_STEP_FUSED && cudaMalloc(&h->ext, extb) != cudaSuccess) {
-        h->ext = nullptr;
-        (void)cudaGetLastError();   // a refused allocation is not an error of the handle
-    }
+    if (phases) lbm::ensure_phases(h);
     *out = h;
     return LBM_OK;
 }

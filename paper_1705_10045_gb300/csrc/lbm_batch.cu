@@ -143,6 +143,31 @@ int upload_descs(lbm_batch* b, long long n) {
                       "batch descriptor copy");
 }
 
+// the slot of the only domain with a step budget; -1 when there are none or several
+int only_active(const lbm_batch* b) {
+    int only = -1;
+    for (size_t d = 0; d < b->doms.size(); ++d)
+        if (b->doms[d] && b->budget[d] > 0) {
+            if (only >= 0) return -1;
+            only = (int)d;
+        }
+    return only;
+}
+
+// A request in which one domain steps takes the single-domain step, whose
+// launches fit the domain (in phases where that is faster) and need no
+// completion counters: the same bits, FP32 126^3 300 -> 181 us a step (178
+// with the best chunk of the persistent launch), 64^3 260 -> 24.
+int step_alone(lbm_batch* b, int d, int n) {
+    lbm_handle* h = b->doms[d];
+    const int m = (int)std::min<long long>(b->budget[d], n);
+    lbm::ensure_phases(h);
+    if (int rc = b->Q == 9 ? lbm::Backend<9>::step(h, m) : lbm::Backend<19>::step(h, m)) return rc;
+    h->steps += m;
+    b->budget[d] -= m;
+    return LBM_OK;
+}
+
 int capture_graph(lbm_batch* b) {
     cudaGraph_t g = nullptr;
     if (int rc = cuda_error(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "graph capture"))
@@ -160,6 +185,7 @@ int capture_graph(lbm_batch* b) {
     b->graph_variant = b->variant;
     b->graph_doms = (int)b->doms.size();
     b->graph_fault = b->fault_item;
+    b->graph_xw = b->xw;
     return LBM_OK;
 }
 
@@ -272,6 +298,7 @@ int lbm_batch_step(lbm_batch* b, int n) {
     }
     if (n == 0) return LBM_OK;
     cudaSetDevice(b->common.device);
+    if (const int only = only_active(b); only >= 0 && b->fault_item < 0) return step_alone(b, only, n);
     if (b->dirty || table_set(b, false) != b->in_table)
         if (int rc = rebuild(b)) return rc;
     // the pinned staging may still feed the previous request's copy
@@ -282,7 +309,7 @@ int lbm_batch_step(lbm_batch* b, int n) {
         const long long m = std::min<long long>(per, n - done);
         if (int rc = upload_descs(b, m)) return rc;
         if (!b->graph || b->graph_items != b->n_items || b->graph_variant != b->variant ||
-            b->graph_doms != (int)b->doms.size() || b->graph_fault != b->fault_item) {
+            b->graph_doms != (int)b->doms.size() || b->graph_fault != b->fault_item || b->graph_xw != b->xw) {
             drop_graph(b);
             if (int rc = capture_graph(b)) return rc;
         }

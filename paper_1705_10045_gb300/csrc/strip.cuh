@@ -70,6 +70,7 @@ template <typename S, typename R, bool WALL> struct Strip {
     int col_m, col_p;       // columns the pushes to x - 1 and x + 1 go to
     bool owns;
     int edge;               // walls beside the column (bit 0 low, bit 1 high)
+    bool edge_strip;        // a column the warp owns lies beside a wall
     Pop<S>* ring;           // the lane's column of the warp's rows in shared memory
     int next_row;           // wrapped index of the row the next load takes
 
@@ -94,6 +95,7 @@ template <typename S, typename R, bool WALL> struct Strip {
         }
         owns = lane >= 2 && lane < 2 + kCols && a < na;
         edge = WALL && p.wall_x ? (a == 0 ? 1 : 0) | (a == na - 1 ? 2 : 0) : 0;
+        edge_strip = WALL && p.wall_x && (a0 == 0 || a0 + kCols >= na);
         col_m = col == 0 ? na - 1 : col - 1;
         col_p = col == na - 1 ? 0 : col + 1;
         next_row = (zb - 2) % nm;
@@ -208,7 +210,8 @@ template <typename S, typename R, bool WALL> struct Strip {
                 else store_pop(dst + k * nn, (unsigned)to, out, t);
             });
         };
-        if (WALL && (gu || gd || edge)) push(std::true_type{});
+        // one instance for the whole warp: lanes apart would run both in turn
+        if (WALL && (gu || gd || edge_strip)) push(std::true_type{});
         else push(std::false_type{});
     }
 
@@ -271,14 +274,14 @@ template <typename S, typename R, bool WALL>
 __global__ void __launch_bounds__(32 * kStripWarps, kStripCtas)
     strip_step_kernel(const S* __restrict__ src, S* __restrict__ dst, const __grid_constant__ KParams<R> p, StripGeom G,
                       Counters* cnt) {
-    using St = Strip<S, R, WALL>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, w = blockIdx.x * kStripWarps + warp;
     const int strip = w % G.strips, zb = G.m_lo + (w / G.strips) * G.chunk;
     if (zb >= G.m_hi) return;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the previous step's stores
+    using St = Strip<S, R, WALL>;
     St s(src, dst, p, cnt, G.na, G.nm, zb, min(zb + G.chunk, G.m_hi), p.step, strip * St::kCols,
          reinterpret_cast<Pop<S>*>(smem_raw + warp * St::kRingBytes));
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the previous step's stores
     s.run();
 }
 
