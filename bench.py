@@ -72,8 +72,8 @@ def _fields():
     return W.pool_boiling_3d(nx=NX, ny=NY, nz=NZ, T=0.8, depth=DEPTH, noise=1e-4, seed=3)
 
 
-KERNEL_SOURCES = ("fused.cuh", "kernels.cuh", "lattice.cuh", "backend.cuh")
-TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "fused_step_kernel_d3q19_fp32.md")
+KERNEL_SOURCES = ("rows.cuh", "strip.cuh", "fused.cuh", "node.cuh", "kernels.cuh", "lattice.cuh", "backend.cuh")
+TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "row_march_kernel_d3q19_fp32.md")
 
 
 def _kernel_source_hash() -> str:
@@ -86,7 +86,7 @@ def _kernel_source_hash() -> str:
 
 
 def _measured_traffic_per_node():
-    """DRAM bytes per node of one fused launch from the committed ncu summary,
+    """DRAM bytes per node of one step launch from the committed ncu summary,
     or None when the kernel sources changed since that capture."""
     if not os.path.exists(TRAFFIC_SUMMARY):
         return None, None
@@ -694,7 +694,7 @@ def main():
         # the 8 field values it needs of its own node (32 B)
         algo_bytes = {"collide_kernel": 4 * 19 * 4 + 8 * 4}.get(top, 4 * 19 * 4)
         achieved = algo_bytes * nn / (prof[top] * 1e-3) / 1e9
-        traffic_per_node, traffic_src = _measured_traffic_per_node() if top == "fused_step_kernel" else (None, None)
+        traffic_per_node, traffic_src = _measured_traffic_per_node() if top == "row_march_kernel" else (None, None)
         value = whole_job_mlups(nn, args.steps, ws, ms * 1e-3)
         line = {
             "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": ws, "steps": args.steps,

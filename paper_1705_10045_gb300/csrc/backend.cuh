@@ -11,6 +11,7 @@
 #include "kernels.cuh"
 #include "output.cuh"
 #include "phases.cuh"
+#include "rows.cuh"
 #include "strip.cuh"
 
 namespace lbm {
@@ -51,9 +52,9 @@ constexpr int kSms = 152;   // SMs of a GB300
 // one drains.  Between ordinary launches of short kernels the step time moved
 // in stairs of 2.05 us (512 x 512 D2Q9: 10.3 us for 8.4 us this way).
 template <typename... P, typename... A>
-void launch_after(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+void launch_after(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -92,42 +93,74 @@ template <> struct BatchShape<19, 2> { static constexpr int TX = 32, TY = 4, NP 
 template <int Q, typename S, typename R> struct Impl {
     static constexpr int TX = FusedTile<Q, R>::TX, TY = FusedTile<Q, R>::TY, NP = FusedTile<Q, R>::NP;
     static constexpr bool SPLIT = FusedTile<Q, R>::SPLIT;
-    // Steps in three phases (phases.cuh): FP64, and D3Q19 domains the march
-    // cannot spread over the SMs (march_us); only where the handle has their
-    // planes.
+    // Steps in three phases (phases.cuh): FP64, and small D3Q19 domains; only
+    // where the handle has their planes.
     static constexpr bool kF64 = std::is_same<S, double>::value;
     static constexpr bool kPhases = kF64 || Q == 19;
     static bool phases(const lbm_handle* h) { return kPhases && h->ext && h->fault_drop <= 0; }
-    static bool wants_phases(int nx, int ny, int nz) {
+    static bool wants_phases(const lbm_params& p) {
         if (kF64) return true;
         if (!kPhases) return false;
         MarchGeom G;
-        G.na = nx;
-        G.nb = ny;
-        G.nm = nz;
-        double t;
-        march_chunk(G, nz, t);
-        return 4.5 + kPhaseNs * 1e-3 * (double)nx * ny * nz < t;
+        G.na = p.nx;
+        G.nb = p.ny;
+        G.nm = p.nz;
+        double t, rows;
+        march_chunk(G, p.nz, t);
+        row_chunk(p, G, p.nz, rows);
+        const double nodes = (double)p.nx * p.ny * p.nz;
+        const double ns = 4.0 * 19 * sizeof(S) * nodes < 110e6 ? kPhaseNsL2 : kPhaseNs;   // both buffers stay in L2
+        return 4.5 + ns * 1e-3 * nodes < std::min(t, rows);
     }
     static int launches(const lbm_handle* h) {
         return h->p.step_kernel == LBM_STEP_THREE_LAUNCH || phases(h) ? 3 : 1;
     }
 
-    // Planes per CTA of the march, and the modelled time t (us) of the launch.
-    // A CTA takes about 4.5 plane times beyond its chunk (ring planes, the
-    // first three planes' moments).  A plane takes kPlane1 us while an SM holds
-    // one CTA and kPlane2 with two (D3Q19, measured: 64^3 in chunks of 8 with
-    // 128 CTAs, 128^3 in chunks of 32 with 256); chunks stay below 65 planes
-    // so that neighbouring tiles of a large domain keep sharing ring lines in
-    // L2.  The chunk with the smallest modelled time avoids nearly empty last
-    // waves: FP32 us per step, two CTAs' worth of planes -> this: 128^3 195 ->
-    // 160 (5 -> 4 chunks), 160 x 128 x 96 188 -> 165, 192^3 569 -> 493.
-    // The phases take 4.5 us and kPhaseNs per node (93 ps FP32, 70 ps FP16),
-    // the march 56 and 49 ps a node where it fills the chip: FP32 32^3 33 -> 7.4,
-    // 48^3 35 -> 12.4, 64^3 35 -> 22.6, 80^3 54 -> 51 by phases; 96^3 75 against
-    // 89 and 128^3 160 against 202 by the march.
+    // D3Q19 in FP32 and FP16 storage has three forms of a step with the same
+    // bits, and takes the one with the smallest modelled time.  Measured us per
+    // step (march / row march / phases): FP32 32^3 33 / - / 7.4, 64^3 35 / 30 /
+    // 22.6, 80^3 54 / 42 / 51, 96^3 75 / 77 / 89, 128^3 160 / 150 / 202, 192^3 493
+    // / 478 / 662, 300^3 1996 / 1705 / -, 448 x 300 x 100 994 / 870 / -, 384 x 384 x
+    // 256 2545 / 2325 / -; FP16 64^3 33 / 24 / 19.4, 96^3 63 / 55 / 68, 128^3 140 /
+    // 124 / 152, 192^3 399 / 343 / 485, 384 x 384 x 256 2020 / 1710 / -.
+    //
+    // Phases: 4.5 us and kPhaseNs (kPhaseNsL2 where both buffers stay in L2) per
+    // node.
+    static constexpr double kPhaseNs = sizeof(S) == 2 ? 0.070 : 0.093, kPhaseNsL2 = sizeof(S) == 2 ? 0.057 : 0.072;
+    // March: planes per CTA, and its modelled time t.  A CTA takes about 4.5
+    // plane times beyond its chunk (ring planes, the first three planes'
+    // moments).  A plane takes kPlane1 us while an SM holds one CTA and kPlane2
+    // with two (64^3 in chunks of 8 with 128 CTAs, 128^3 in chunks of 32 with
+    // 256), 6 % more where CTAs of several waves run out of step; chunks stay
+    // below 65 planes so that neighbouring tiles keep sharing ring lines in L2.
+    // The chunk with the smallest modelled time avoids nearly empty last waves:
+    // FP32, two CTAs' worth of planes -> this: 128^3 195 -> 160 (5 -> 4 chunks),
+    // 160 x 128 x 96 188 -> 165, 192^3 569 -> 493.
     static constexpr double kPlane1 = sizeof(S) == 2 ? 2.6 : 2.7, kPlane2 = sizeof(S) == 2 ? 3.85 : 4.4;
-    static constexpr double kPhaseNs = sizeof(S) == 2 ? 0.070 : 0.093;
+    // Row march (rows.cuh): planes per CTA, and its modelled time t: one CTA per
+    // SM, (planes + 2.5) times kRowPlane us a wave.  0 where it does not run:
+    // walls on x, rows that are no multiple of 16 bytes.
+    static constexpr bool kRows = Q == 19 && !kF64;
+    static constexpr double kRowPlane = sizeof(S) == 2 ? 3.1 : 2.25;
+    static int row_chunk(const lbm_params& p, const MarchGeom& G, int len, double& t) {
+        int best = 0;
+        t = 1e30;
+        if constexpr (kRows) {
+            if (p.wall_x || G.na % (8 / (int)sizeof(S)) != 0) return 0;
+            const long long tiles = (long long)strip_count(G.na) * ((G.nb + RowShape<S>::TY - 1) / RowShape<S>::TY);
+            for (int n = (len + 63) / 64; n <= len; ++n) {
+                const int c = (len + n - 1) / n;
+                if ((len + c - 1) / c != n) continue;
+                const double tn = (c + 2.5) * kRowPlane * (double)((tiles * n + kSms - 1) / kSms);
+                if (tn < t) {
+                    t = tn;
+                    best = c;
+                }
+            }
+        }
+        return best;
+    }
+
     static int march_chunk(const MarchGeom& G, int len, double& t) {
         const long long tiles = (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY);
         const int few = (len + 63) / 64;   // chunks per column of tiles, at least
@@ -137,7 +170,8 @@ template <int Q, typename S, typename R> struct Impl {
             const int c = (len + n - 1) / n;
             if ((len + c - 1) / c != n) continue;
             const long long ctas = tiles * n, full = ctas / (2 * kSms), rest = ctas % (2 * kSms);
-            const double tn = (c + 4.5) * ((double)full * kPlane2 + (rest > kSms ? kPlane2 : (rest ? kPlane1 : 0.0)));
+            const double tn = (c + 4.5) * ((double)full * kPlane2 + (rest > kSms ? kPlane2 : (rest ? kPlane1 : 0.0))) *
+                              (full ? 1.06 : 1.0);
             if (tn < t) {
                 t = tn;
                 best = c;
@@ -166,6 +200,15 @@ template <int Q, typename S, typename R> struct Impl {
         double t;
         G.chunk = march_chunk(G, G.m_hi - G.m_lo, t);
         return G;
+    }
+
+    // name of the kernel of a step in one launch
+    static const char* single_name(const lbm_handle* h) {
+        if (kStrips) return "strip_step_kernel";
+        const MarchGeom G = geometry(h);
+        double rows, march;
+        march_chunk(G, G.m_hi - G.m_lo, march);
+        return row_chunk(h->p, G, G.m_hi - G.m_lo, rows) > 0 && rows < march ? "row_march_kernel" : "fused_step_kernel";
     }
 
     static void launch_fused(lbm_handle* h, const KParams<R>& kp) {
@@ -235,6 +278,27 @@ template <int Q, typename S, typename R> struct Impl {
                 }
                 launch_after(kern, grid, 32 * kStripWarps, smem, h->stream, src, dst, kp, g, (Counters*)h->cnt);
                 return;
+            }
+        }
+        if constexpr (kRows) {
+            double t;
+            MarchGeom g = G;
+            if (h->fault_drop <= 0 && (g.chunk = row_chunk(h->p, G, G.m_hi - G.m_lo, t)) > 0) {
+                double march;
+                march_chunk(G, G.m_hi - G.m_lo, march);
+                if (t < march) {
+                    using Sh = RowShape<S>;
+                    constexpr size_t bytes = RowMarch<S, R, Sh::TY, Sh::AHEAD, true>::kBytes;
+                    auto kern = h->p.wall || h->p.wall_y ? row_march_kernel<S, R, true> : row_march_kernel<S, R, false>;
+                    if (!h->rows_ready) {
+                        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                        h->rows_ready = true;
+                    }
+                    launch_after(kern, dim3(strip_count(G.na), (G.nb + Sh::TY - 1) / Sh::TY,
+                                            (G.m_hi - G.m_lo + g.chunk - 1) / g.chunk),
+                                 32 * (Sh::TY + 4), bytes, h->stream, src, dst, kp, g, (Counters*)h->cnt);
+                    return;
+                }
             }
         }
         const size_t smem = FusedShape<TX, TY, SPLIT>::template smem_bytes<R>();
@@ -567,7 +631,11 @@ template <int Q> const char* Backend<Q>::launch_name(const lbm_handle* h, int j)
     static const char* phase[] = {"phase_moments_kernel", "phase_force_kernel", "phase_collide_kernel"};
     if (launches(h) == 3) return j >= 0 && j < 3 ? phase[j] : "";
     if (j != 0) return "";
-    return Q == 9 && h->p.storage != LBM_STORE_FP64 ? "strip_step_kernel" : "fused_step_kernel";
+    switch (h->p.storage) {
+        case LBM_STORE_FP64: return Impl<Q, double, double>::single_name(h);
+        case LBM_STORE_FP32: return Impl<Q, float, float>::single_name(h);
+        default: return Impl<Q, __half, float>::single_name(h);
+    }
 }
 template <int Q> int Backend<Q>::launches(const lbm_handle* h) { LBM_DISPATCH(h, launches(h)); }
 template <int Q> int Backend<Q>::init(lbm_handle* h, const double* rho, const double* u, const double* eps) {
@@ -611,8 +679,8 @@ template <int Q> size_t Backend<Q>::phase_bytes(const lbm_params* p) {
     const size_t planes = (size_t)X_COUNT * (size_t)p->nx * p->ny * p->nz;
     switch (p->storage) {
         case LBM_STORE_FP64: return planes * sizeof(double);
-        case LBM_STORE_FP32: return Impl<Q, float, float>::wants_phases(p->nx, p->ny, p->nz) ? planes * sizeof(float) : 0;
-        default: return Impl<Q, __half, float>::wants_phases(p->nx, p->ny, p->nz) ? planes * sizeof(float) : 0;
+        case LBM_STORE_FP32: return Impl<Q, float, float>::wants_phases(*p) ? planes * sizeof(float) : 0;
+        default: return Impl<Q, __half, float>::wants_phases(*p) ? planes * sizeof(float) : 0;
     }
 }
 

@@ -21,8 +21,8 @@
 // In FP32 and FP16 storage the populations are read twice and the fields add
 // traffic (about 93 ps a node against the march's 56), but every node has its
 // own thread and no plane waits for another: domains too small to fill 152 SMs
-// with marching CTAs step faster this way (the rule and figures stand at
-// march_chunk in backend.cuh).
+// with marching CTAs step faster this way (the rule and figures stand in
+// backend.cuh).
 #pragma once
 
 #include "node.cuh"
