@@ -1,9 +1,12 @@
 // Launch sequences of the liblbm back end for one lattice, for every storage
 // format.  Included once per lattice by lbm_d2q9.cu and lbm_d3q19.cu.
 //
-// A time step is either the fused single launch (fused_step_kernel, the
-// default) or the three-launch form fields -> force -> collide, kept as a
-// second, independently structured statement of the same step.
+// A time step takes one of four forms that round alike and so leave the same
+// bits: strips of columns (D2Q9 FP32 and FP16, strip.cuh), rows of columns
+// (rows.cuh) or the producer/consumer march (fused.cuh) for D3Q19, and three
+// launches over all nodes (FP64 and small D3Q19 domains, phases.cuh).  The
+// form fields -> force -> collide (LBM_STEP_THREE_LAUNCH) is kept as a second,
+// independently structured statement of the same step.
 #pragma once
 
 #include "fused.cuh"
@@ -161,6 +164,14 @@ template <int Q, typename S, typename R> struct Impl {
         return best;
     }
 
+    // planes per CTA of the row march where it is modelled faster than the march, else 0
+    static int rows_instead(const lbm_params& p, const MarchGeom& G) {
+        double rows, march;
+        const int c = row_chunk(p, G, G.m_hi - G.m_lo, rows);
+        march_chunk(G, G.m_hi - G.m_lo, march);
+        return rows < march ? c : 0;
+    }
+
     static int march_chunk(const MarchGeom& G, int len, double& t) {
         const long long tiles = (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY);
         const int few = (len + 63) / 64;   // chunks per column of tiles, at least
@@ -205,10 +216,7 @@ template <int Q, typename S, typename R> struct Impl {
     // name of the kernel of a step in one launch
     static const char* single_name(const lbm_handle* h) {
         if (kStrips) return "strip_step_kernel";
-        const MarchGeom G = geometry(h);
-        double rows, march;
-        march_chunk(G, G.m_hi - G.m_lo, march);
-        return row_chunk(h->p, G, G.m_hi - G.m_lo, rows) > 0 && rows < march ? "row_march_kernel" : "fused_step_kernel";
+        return rows_instead(h->p, geometry(h)) > 0 ? "row_march_kernel" : "fused_step_kernel";
     }
 
     static void launch_fused(lbm_handle* h, const KParams<R>& kp) {
@@ -259,6 +267,11 @@ template <int Q, typename S, typename R> struct Impl {
 
     // the fused step over the planes of G, src -> dst (no buffer swap)
     static void launch_fused_range(lbm_handle* h, const KParams<R>& kp, const MarchGeom& G, const S* src, S* dst) {
+        Counters* cnt = (Counters*)h->cnt;
+        if (h->fault_drop > 0) {   // fault-injection test hook (lbm_test_drop_handoff)
+            launch_fault(h, kp, G, src, dst);
+            return;
+        }
         if constexpr (kPhases) {
             if (phases(h)) {
                 for (int j = 0; j < 3; ++j) launch_phase(h, kp, G, src, dst, j);
@@ -266,60 +279,49 @@ template <int Q, typename S, typename R> struct Impl {
             }
         }
         if constexpr (kStrips) {
-            if (h->fault_drop <= 0) {
-                const StripGeom g = strip_geometry(G);
-                const long long warps = (long long)g.strips * ((g.m_hi - g.m_lo + g.chunk - 1) / g.chunk);
-                const unsigned grid = grid_for(warps, kStripWarps);
-                auto kern = h->p.wall || h->p.wall_x ? strip_step_kernel<S, R, true> : strip_step_kernel<S, R, false>;
-                const size_t smem = kStripWarps * Strip<S, R, false>::kRingBytes;
-                if (!h->fused_ready) {
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                    h->fused_ready = true;
-                }
-                launch_after(kern, grid, 32 * kStripWarps, smem, h->stream, src, dst, kp, g, (Counters*)h->cnt);
-                return;
-            }
-        }
-        if constexpr (kRows) {
-            double t;
-            MarchGeom g = G;
-            if (h->fault_drop <= 0 && (g.chunk = row_chunk(h->p, G, G.m_hi - G.m_lo, t)) > 0) {
-                double march;
-                march_chunk(G, G.m_hi - G.m_lo, march);
-                if (t < march) {
+            const StripGeom g = strip_geometry(G);
+            const long long warps = (long long)g.strips * ((g.m_hi - g.m_lo + g.chunk - 1) / g.chunk);
+            auto kern = h->p.wall || h->p.wall_x ? strip_step_kernel<S, R, true> : strip_step_kernel<S, R, false>;
+            const size_t smem = kStripWarps * Strip<S, R, false>::kRingBytes;
+            allow_smem(kern, smem, h->fused_ready);
+            launch_after(kern, grid_for(warps, kStripWarps), 32 * kStripWarps, smem, h->stream, src, dst, kp, g, cnt);
+        } else {
+            if constexpr (kRows) {
+                MarchGeom g = G;
+                if ((g.chunk = rows_instead(h->p, G)) > 0) {
                     using Sh = RowShape<S>;
-                    constexpr size_t bytes = RowMarch<S, R, Sh::TY, Sh::AHEAD, true>::kBytes;
+                    constexpr size_t smem = RowMarch<S, R, Sh::TY, Sh::AHEAD, true>::kBytes;
                     auto kern = h->p.wall || h->p.wall_y ? row_march_kernel<S, R, true> : row_march_kernel<S, R, false>;
-                    if (!h->rows_ready) {
-                        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-                        h->rows_ready = true;
-                    }
+                    allow_smem(kern, smem, h->rows_ready);
                     launch_after(kern, dim3(strip_count(G.na), (G.nb + Sh::TY - 1) / Sh::TY,
                                             (G.m_hi - G.m_lo + g.chunk - 1) / g.chunk),
-                                 32 * (Sh::TY + 4), bytes, h->stream, src, dst, kp, g, (Counters*)h->cnt);
+                                 32 * (Sh::TY + 4), smem, h->stream, src, dst, kp, g, cnt);
                     return;
                 }
             }
+            const size_t smem = FusedShape<TX, TY, SPLIT>::template smem_bytes<R>();
+            const bool xw = h->p.wall_x || (Q == 19 && h->p.wall_y);
+            auto kern = xw ? fused_step_kernel<Q, S, R, TX, TY, NP, true, SPLIT>
+                           : fused_step_kernel<Q, S, R, TX, TY, NP, false, SPLIT>;
+            allow_smem(kern, smem, h->fused_ready);
+            const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
+            kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, cnt);
         }
+    }
+    // raise a kernel's shared-memory limit, once per handle
+    template <typename K> static void allow_smem(K kern, size_t smem, bool& ready) {
+        if (!ready) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        ready = true;
+    }
+    // the march with the fault-injection hook; long chunks, so that the first
+    // CTA marches over the plane
+    static void launch_fault(lbm_handle* h, const KParams<R>& kp, MarchGeom G, const S* src, S* dst) {
+        G.chunk = std::min(64, G.m_hi - G.m_lo);
         const size_t smem = FusedShape<TX, TY, SPLIT>::template smem_bytes<R>();
-        const bool xw = h->p.wall_x || (Q == 19 && h->p.wall_y);
-        auto kern = xw ? fused_step_kernel<Q, S, R, TX, TY, NP, true, SPLIT>
-                       : fused_step_kernel<Q, S, R, TX, TY, NP, false, SPLIT>;
-        if (!h->fused_ready) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            h->fused_ready = true;
-        }
-        dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
-        if (h->fault_drop > 0) {   // fault-injection test hook (lbm_test_drop_handoff)
-            MarchGeom F = G;       // long chunks, so that the first CTA marches over the plane
-            F.chunk = std::min(64, G.m_hi - G.m_lo);
-            grid.z = (G.m_hi - G.m_lo + F.chunk - 1) / F.chunk;
-            auto fk = fused_step_fault_kernel<Q, S, R, TX, TY, NP, SPLIT>;
-            cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            fk<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, F, (Counters*)h->cnt, h->fault_drop - 1);
-        } else {
-            kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, (Counters*)h->cnt);
-        }
+        const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
+        auto kern = fused_step_fault_kernel<Q, S, R, TX, TY, NP, SPLIT>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, (Counters*)h->cnt, h->fault_drop - 1);
     }
 
     // planes [first, first + count) of the step lbm_step_begin opened: it has

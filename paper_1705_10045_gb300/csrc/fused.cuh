@@ -23,10 +23,13 @@
 // plane c when C(c) has read its buffers, which the producers wait for before
 // overwriting them.  Neither role waits for the other's whole iteration, so a
 // slow plane on one side does not stall the other.  A named barrier orders M
-// before F, and F before the next M, inside the producer warps.  Ring nodes are recomputed by neighbouring
-// CTAs from L2 rather than exchanged.  D2Q9 runs the same code as a lattice
-// with one y node: its lattice y axis is the march axis and its tile is
-// TX x 1.
+// before F, and F before the next M, inside the producer warps.  Ring nodes
+// are recomputed by neighbouring CTAs from L2 rather than exchanged.  D2Q9
+// runs the same code as a lattice with one y node: its lattice y axis is the
+// march axis and its tile is TX x 1 (FP64 without memory for its phases, and
+// the fault-injection form; D2Q9 otherwise steps strips, strip.cuh).  Batches
+// of D3Q19 domains run it, and the single domains for which backend.cuh
+// models it faster than rows.cuh and phases.cuh.
 //
 // Index arithmetic is kept out of the inner loops: the wrapped ring
 // coordinates of a CTA are tabulated once in shared memory, buffer slots come

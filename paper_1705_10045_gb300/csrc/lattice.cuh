@@ -190,8 +190,8 @@ template <> struct Store<float, float> {
 // mantissa bits of the FP32 value and rounding toward zero rounds the
 // magnitude up with probability equal to the discarded fraction (unbiased
 // for FP16-normal values).  The conversion drops the 13 low bits itself.
-// The _raw forms move the stored, shifted values as they are (kShifted: a
-// kernel may do its arithmetic on shifted values and skip the shifts).
+// kShifted: a kernel may do its arithmetic on the stored, shifted values and
+// skip the shifts (word, lo, hi, add_*, sub_lo, store2_raw).
 template <> struct Store<__half, float> {
     static constexpr bool kStochastic = true, kShifted = true;
     __device__ static float load(const __half* p, size_t i, float shift) {
@@ -200,10 +200,6 @@ template <> struct Store<__half, float> {
     __device__ static void unpack(unsigned w, float sN, float sG, float& a, float& b) {
         a = __half2float(__ushort_as_half((unsigned short)(w & 0xFFFFu))) + sN;
         b = __half2float(__ushort_as_half((unsigned short)(w >> 16))) + sG;
-    }
-    __device__ static void unpack_raw(unsigned w, float& a, float& b) {
-        a = __half2float(__ushort_as_half((unsigned short)(w & 0xFFFFu)));
-        b = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
     }
     __device__ static unsigned word(const __half* p, size_t i) { return __ldg(reinterpret_cast<const unsigned*>(p) + i); }
     __device__ static unsigned word_last(const __half* p, size_t i) {
@@ -236,7 +232,6 @@ template <> struct Store<__half, float> {
     __device__ static void load2_last_coh(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
         unpack(word_last_coh(p, i), sN, sG, a, b);
     }
-    __device__ static void load2_raw(const __half* p, size_t i, float& a, float& b) { unpack_raw(word(p, i), a, b); }
     // the halves of a pair word widened, and sums with one half rounded once in
     // FP32 (mixed-precision add / sub: a half widens to FP32 exactly, so these
     // equal widening first, in one instruction fewer)
@@ -256,15 +251,6 @@ template <> struct Store<__half, float> {
         float r;
         asm("sub.rn.f32.f16 %0, %1, %2;" : "=f"(r) : "h"((unsigned short)(w & 0xFFFFu)), "f"(acc));
         return r;
-    }
-    __device__ static void load2_last_raw(const __half* p, size_t i, float& a, float& b) {
-        unpack_raw(word_last(p, i), a, b);
-    }
-    __device__ static void load2_coh_raw(const __half* p, size_t i, float& a, float& b) {
-        unpack_raw(word_coh(p, i), a, b);
-    }
-    __device__ static void load2_last_coh_raw(const __half* p, size_t i, float& a, float& b) {
-        unpack_raw(word_last_coh(p, i), a, b);
     }
     // both halves rounded stochastically by one packed conversion (g_k in the
     // high half) with the random word t; a, b already shifted

@@ -19,11 +19,14 @@
 // L2).  The 16-byte copies bypass L1, which is what is left of the shared
 // memory; 8- and 4-byte copies through it gave 3530 and 1890 us.
 //
-// What bounds it: DRAM latency and traffic.  Against the producer/consumer
+// What bounds it: instructions and the barrier a plane.  Against the producer/consumer
 // march of fused.cuh, which reads every node's pairs twice (the second time
 // partly from DRAM) and holds its loads in flight in registers and L1, 384 x
 // 384 x 256 in us per step: FP32 2545 -> 2325 (4.94 TB/s of 304 B per node,
-// 0.73 of the measured copy bandwidth), FP16 storage 2020 -> 1710.
+// 0.73 of the measured copy bandwidth), FP16 storage 2020 -> 1720.  DRAM reads
+// are 1.01 times the populations (march: 1.24 to 1.30); the wait at the
+// barrier comes first now (1.6 cycles per instruction), issue is 50 % busy in
+// FP32 and 68 % in FP16.
 #pragma once
 
 #include "fused.cuh"
@@ -274,9 +277,18 @@ __global__ void __launch_bounds__(32 * (RowShape<S>::TY + 4), 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int zb = G.m_lo + blockIdx.z * G.chunk;
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the previous step's stores
-    RowMarch<S, R, Sh::TY, Sh::AHEAD, WALL> r(src, dst, p, cnt, G, blockIdx.x * kStripCols, blockIdx.y * Sh::TY, zb,
-                                              min(zb + G.chunk, G.m_hi), p.step, smem_raw);
-    r.run();
+    const int ze = min(zb + G.chunk, G.m_hi), a0 = blockIdx.x * kStripCols, b0 = blockIdx.y * Sh::TY;
+    // a CTA none of whose ring nodes lies beyond a wall takes the periodic code
+    // (384 x 384 x 256 between walls on z: FP32 2377 -> 2340 us, FP16 1851 -> 1790;
+    // periodic 2325 and 1720)
+    const bool walled = WALL && ((p.wall && (zb < 2 || ze + 2 > G.nm)) || (p.wall_y && (b0 < 2 || b0 + Sh::TY + 2 > G.nb)));
+    if (WALL && walled) {
+        RowMarch<S, R, Sh::TY, Sh::AHEAD, true> r(src, dst, p, cnt, G, a0, b0, zb, ze, p.step, smem_raw);
+        r.run();
+    } else {
+        RowMarch<S, R, Sh::TY, Sh::AHEAD, false> r(src, dst, p, cnt, G, a0, b0, zb, ze, p.step, smem_raw);
+        r.run();
+    }
 }
 
 }  // namespace lbm
