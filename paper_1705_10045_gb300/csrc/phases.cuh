@@ -23,6 +23,11 @@
 // own thread and no plane waits for another: domains too small to fill 152 SMs
 // with marching CTAs step faster this way (the rule and figures stand in
 // backend.cuh).
+//
+// Each launch starts while the one before it still writes (backend.cuh,
+// launch_after), so what a launch reads is not constant for its whole life:
+// populations and fields come through coherent loads behind
+// griddepcontrol.wait, never through const __restrict__ pointers.
 #pragma once
 
 #include "node.cuh"
@@ -58,8 +63,8 @@ template <int Q, typename S, typename R> struct Phase {
 };
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict__ src, R* __restrict__ fld,
-                                                            R* __restrict__ ext, const __grid_constant__ KParams<R> p,
+__global__ void __launch_bounds__(128) phase_moments_kernel(const S* src, R* fld, R* ext,
+                                                            const __grid_constant__ KParams<R> p,
                                                             PhaseGeom G, Counters* cnt) {
     using Math = NodeMath<Q, S, R>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -68,7 +73,7 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict_
     const size_t nn = (size_t)p.nn;
     Pop<S> f[Q];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) f[k] = load_pop<false>(src + 2 * ((size_t)k * nn), (size_t)n);
+    for (int k = 0; k < Q; ++k) f[k] = load_pop<true>(src + 2 * ((size_t)k * nn), (size_t)n);
     const Moments<R> o = Math::moments(f, p);
     const R inv = R(1) / o.rho;
     const R T = o.E / (o.rho * p.c_v), P = eos_pressure(p, o.rho, T);
@@ -92,7 +97,7 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* __restrict_
 }
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, const __grid_constant__ KParams<R> p, PhaseGeom G) {
+__global__ void __launch_bounds__(128) phase_force_kernel(R* fld, const __grid_constant__ KParams<R> p, PhaseGeom G) {
     using Ph = Phase<Q, S, R>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int n = Ph::node(G);
@@ -115,8 +120,7 @@ __global__ void __launch_bounds__(128) phase_force_kernel(R* __restrict__ fld, c
 }
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_collide_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                            const R* __restrict__ fld, const R* __restrict__ ext,
+__global__ void __launch_bounds__(128) phase_collide_kernel(const S* src, S* dst, const R* fld, const R* ext,
                                                             const __grid_constant__ KParams<R> p, PhaseGeom G) {
     using Ph = Phase<Q, S, R>;
     using Math = NodeMath<Q, S, R>;
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(128) phase_collide_kernel(const S* __restrict_
     const typename Ph::Steps s(p, n);
     Pop<S> f[Q];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) f[k] = load_pop<false>(src + 2 * ((size_t)k * nn), (size_t)n);
+    for (int k = 0; k < Q; ++k) f[k] = load_pop<true>(src + 2 * ((size_t)k * nn), (size_t)n);
     const R rho = fld[F_RHO * nn + n], T = fld[F_T * nn + n];
     R u[3] = {0, 0, 0}, dv[3] = {0, 0, 0};   // in march order (a, b, m)
 #pragma unroll

@@ -44,8 +44,8 @@ template <typename S, typename R, int TY, int AHEAD, bool WALL> struct RowMarch 
     static constexpr size_t kBytes = kPopBytes + sizeof(R) * (size_t)(4 * kRows * kStride + 3 * 2 * kRows * 32);
     static_assert(kBytes <= 227 * 1024, "shared memory");
 
-    const Pop<S>* __restrict__ src;
-    Pop<S>* __restrict__ dst;
+    const Pop<S>* src;   // written by the previous launch until griddepcontrol.wait: not __restrict__
+    Pop<S>* dst;
     const KParams<R>& p;
     Counters* cnt;
     size_t nn;
@@ -271,7 +271,7 @@ template <> struct RowShape<__half> { static constexpr int TY = 16, AHEAD = 2; }
 // planes.  WALL: the domain has walls on y or z (x is periodic).
 template <typename S, typename R, bool WALL>
 __global__ void __launch_bounds__(32 * (RowShape<S>::TY + 4), 1)
-    row_march_kernel(const S* __restrict__ src, S* __restrict__ dst, const __grid_constant__ KParams<R> p, MarchGeom G,
+    row_march_kernel(const S* src, S* dst, const __grid_constant__ KParams<R> p, MarchGeom G,
                      Counters* cnt) {
     using Sh = RowShape<S>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -59,8 +59,8 @@ template <typename S, typename R, bool WALL> struct Strip {
     static constexpr size_t kRingBytes = sizeof(Pop<S>) * Q * 32 * kRows;   // per warp
     using Math = NodeMath<9, S, R>;
 
-    const Pop<S>* __restrict__ src;
-    Pop<S>* __restrict__ dst;
+    const Pop<S>* src;   // written by the previous launch until griddepcontrol.wait: not __restrict__
+    Pop<S>* dst;
     const KParams<R>& p;
     Counters* cnt;
     size_t nn;
@@ -272,7 +272,7 @@ inline int strip_rows(int strips, int len, int sms) {
 
 template <typename S, typename R, bool WALL>
 __global__ void __launch_bounds__(32 * kStripWarps, kStripCtas)
-    strip_step_kernel(const S* __restrict__ src, S* __restrict__ dst, const __grid_constant__ KParams<R> p, StripGeom G,
+    strip_step_kernel(const S* src, S* dst, const __grid_constant__ KParams<R> p, StripGeom G,
                       Counters* cnt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, w = blockIdx.x * kStripWarps + warp;
