@@ -236,10 +236,7 @@ typedef struct lbm_batch lbm_batch;
 
 /* Device memory in bytes a domain with parameters *p needs (admission control),
  * counting the staging planes it keeps once fields have moved between it and
- * host memory (lbm_init or lbm_moments with host pointers).  A handle from
- * lbm_create that steps in three fused-form kernels (FP64, small D3Q19 domains)
- * takes two more fields when there is memory for them; a batch's domains do
- * not. */
+ * host memory (lbm_init or lbm_moments with host pointers). */
 size_t lbm_domain_bytes(const lbm_params* p);
 
 /* New empty batch for common->lattice and common->storage on common->device.

@@ -96,11 +96,10 @@ template <> struct BatchShape<19, 2> { static constexpr int TX = 32, TY = 4, NP 
 template <int Q, typename S, typename R> struct Impl {
     static constexpr int TX = FusedTile<Q, R>::TX, TY = FusedTile<Q, R>::TY, NP = FusedTile<Q, R>::NP;
     static constexpr bool SPLIT = FusedTile<Q, R>::SPLIT;
-    // Steps in three phases (phases.cuh): FP64, and small D3Q19 domains; only
-    // where the handle has their planes.
+    // Steps in three phases (phases.cuh): FP64, and small D3Q19 domains.
     static constexpr bool kF64 = std::is_same<S, double>::value;
     static constexpr bool kPhases = kF64 || Q == 19;
-    static bool phases(const lbm_handle* h) { return kPhases && h->ext && h->fault_drop <= 0; }
+    static bool phases(const lbm_handle* h) { return kPhases && h->phases && h->fault_drop <= 0; }
     static bool wants_phases(const lbm_params& p) {
         if (kF64) return true;
         if (!kPhases) return false;
@@ -259,10 +258,9 @@ template <int Q, typename S, typename R> struct Impl {
         }
         const unsigned grid = grid_for((long long)g.count * g.plane_n, 128);
         R* fld = (R*)h->fld;
-        R* ext = (R*)h->ext;
-        if (j == 0) launch_after(phase_moments_kernel<Q, S, R>, grid, 128, 0, h->stream, src, fld, ext, kp, g, (Counters*)h->cnt);
+        if (j == 0) launch_after(phase_moments_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, kp, g, (Counters*)h->cnt);
         if (j == 1) launch_after(phase_force_kernel<Q, S, R>, grid, 128, 0, h->stream, fld, kp, g);
-        if (j == 2) launch_after(phase_collide_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, ext, kp, g);
+        if (j == 2) launch_after(phase_collide_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, kp, g);
     }
 
     // the fused step over the planes of G, src -> dst (no buffer swap)
@@ -273,12 +271,14 @@ template <int Q, typename S, typename R> struct Impl {
             return;
         }
         if constexpr (kPhases) {
-            if (phases(h)) {
+            if (kF64 || phases(h)) {
                 for (int j = 0; j < 3; ++j) launch_phase(h, kp, G, src, dst, j);
                 return;
             }
         }
-        if constexpr (kStrips) {
+        if constexpr (kF64) {
+            return;
+        } else if constexpr (kStrips) {
             const StripGeom g = strip_geometry(G);
             const long long warps = (long long)g.strips * ((g.m_hi - g.m_lo + g.chunk - 1) / g.chunk);
             auto kern = h->p.wall || h->p.wall_x ? strip_step_kernel<S, R, true> : strip_step_kernel<S, R, false>;
@@ -677,12 +677,11 @@ template <int Q> size_t Backend<Q>::desc_bytes(int storage) {
 template <int Q> size_t Backend<Q>::field_bytes(int storage) {
     return (size_t)F_COUNT * (storage == LBM_STORE_FP64 ? sizeof(double) : sizeof(float));
 }
-template <int Q> size_t Backend<Q>::phase_bytes(const lbm_params* p) {
-    const size_t planes = (size_t)X_COUNT * (size_t)p->nx * p->ny * p->nz;
+template <int Q> bool Backend<Q>::wants_phases(const lbm_params* p) {
     switch (p->storage) {
-        case LBM_STORE_FP64: return planes * sizeof(double);
-        case LBM_STORE_FP32: return Impl<Q, float, float>::wants_phases(*p) ? planes * sizeof(float) : 0;
-        default: return Impl<Q, __half, float>::wants_phases(*p) ? planes * sizeof(float) : 0;
+        case LBM_STORE_FP64: return Impl<Q, double, double>::wants_phases(*p);
+        case LBM_STORE_FP32: return Impl<Q, float, float>::wants_phases(*p);
+        default: return Impl<Q, __half, float>::wants_phases(*p);
     }
 }
 

@@ -17,7 +17,7 @@ struct lbm_handle {
     void* pop[2] = {nullptr, nullptr};   // ping-pong population buffers, 2Q planes each
     int cur = 0;                // buffer holding the current state
     void* fld = nullptr;        // field planes (arithmetic type)
-    void* ext = nullptr;        // field planes of a step in phases (null: the fused step)
+    bool phases = false;        // steps in three phases
     void* cnt = nullptr;        // lbm::Counters on the device
     double* partials = nullptr; // reduction scratch: block partials + 8 results
     double* staging = nullptr;  // (D + 3) planes of doubles for host transfers, allocated on demand
@@ -88,11 +88,6 @@ struct HandleLayout {
     size_t pop1 = 0, fld = 0, cnt = 0, partials = 0, bytes = 0;
     explicit HandleLayout(const lbm_params& p);
 };
-// lbm_create; phases: also allocate the field planes of a step in three phases,
-// for domains that step so (without them, or when there is no memory left for
-// them, those take the fused march, as the domains of a batch do together)
-int create_handle(const lbm_params* p, lbm_handle** out, bool phases);
-void ensure_phases(lbm_handle* h);   // those field planes, if the domain steps so and there is memory
 int ensure_staging(lbm_handle* h);   // the handle's host-transfer buffer, allocated on first use
 // Conservation sums of nodes [i0, i0 + n) through `partials` (block partials,
 // then 8 results): out[0..4] the sums, out[5] clamped and out[6] bad nodes.
@@ -121,7 +116,7 @@ template <int Q> struct Backend {
     // sums over nodes [i0, i0 + n): 5 sums and 3 counters into device memory
     static int reduce(lbm_handle* h, long long i0, long long n, double* partials, double* out_dev);
     static size_t field_bytes(int storage);
-    static size_t phase_bytes(const lbm_params* p);   // extra field planes, 0 when the domain does not step in phases
+    static bool wants_phases(const lbm_params* p);
     // batches: shapes, work table, descriptors, and one request (clear, the
     // persistent launch, and the descriptor advance when `advance`)
     static int batch_variants();

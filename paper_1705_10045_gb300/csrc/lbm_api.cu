@@ -53,15 +53,6 @@ int ensure_staging(lbm_handle* h) {
                       "staging allocation");
 }
 
-void ensure_phases(lbm_handle* h) {
-    if (h->ext || h->p.step_kernel != LBM_STEP_FUSED) return;
-    const size_t bytes = h->Q == 9 ? Backend<9>::phase_bytes(&h->p) : Backend<19>::phase_bytes(&h->p);
-    if (bytes && cudaMalloc(&h->ext, bytes) != cudaSuccess) {
-        h->ext = nullptr;
-        (void)cudaGetLastError();   // a refused allocation is not an error of the handle
-    }
-}
-
 }  // namespace lbm
 
 using lbm::cuda_error;
@@ -285,12 +276,6 @@ void lbm_default_params(lbm_params* p) {
 
 int lbm_create(const lbm_params* p, lbm_handle** out) {
     lbm::TraceRange trace_("lbm_create");
-    return lbm::create_handle(p, out, true);
-}
-
-}  // extern "C"
-
-int lbm::create_handle(const lbm_params* p, lbm_handle** out, bool phases) {
     if (!p || !out) {
         set_error("lbm_create: null argument");
         return LBM_ERR_INVALID_ARG;
@@ -372,12 +357,11 @@ int lbm::create_handle(const lbm_params* p, lbm_handle** out, bool phases) {
         lbm_destroy(h);
         return rc;
     }
-    if (phases) lbm::ensure_phases(h);
+    h->phases = p->step_kernel == LBM_STEP_FUSED &&
+                (h->Q == 9 ? lbm::Backend<9>::wants_phases(p) : lbm::Backend<19>::wants_phases(p));
     *out = h;
     return LBM_OK;
 }
-
-extern "C" {
 
 int lbm_coexistence(double T, double* rho_v, double* rho_l) {
     if (!rho_v || !rho_l || !lbm::coexistence(T, rho_v, rho_l)) {
@@ -643,7 +627,6 @@ void lbm_destroy(lbm_handle* h) {
     DeviceGuard dg(h->p.device);
     if (h->stream) cudaStreamSynchronize(h->stream);
     cudaFree(h->slab);
-    cudaFree(h->ext);
     cudaFree(h->staging);
     cudaFree(h->coex);
     cudaFreeHost(h->bounce);

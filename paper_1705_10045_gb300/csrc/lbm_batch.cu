@@ -161,7 +161,6 @@ int only_active(const lbm_batch* b) {
 int step_alone(lbm_batch* b, int d, int n) {
     lbm_handle* h = b->doms[d];
     const int m = (int)std::min<long long>(b->budget[d], n);
-    lbm::ensure_phases(h);
     if (int rc = b->Q == 9 ? lbm::Backend<9>::step(h, m) : lbm::Backend<19>::step(h, m)) return rc;
     h->steps += m;
     b->budget[d] -= m;
@@ -260,7 +259,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_params* p, const double* rho, const do
     q.device = b->common.device;
     q.step_kernel = LBM_STEP_FUSED;
     lbm_handle* h = nullptr;
-    if (int rc = lbm::create_handle(&q, &h, false)) return rc;
+    if (int rc = lbm_create(&q, &h)) return rc;
     if (int rc = lbm_init(h, rho, u, eps, mem)) {
         lbm_destroy(h);
         return rc;

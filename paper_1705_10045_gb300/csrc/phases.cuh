@@ -1,5 +1,5 @@
 // One time step as three launches over all nodes, each value formed once:
-//   phase_moments   rho, u, T, P, E, Phi of every node
+//   phase_moments   rho, u, T, Phi (fields) and E, P (kept where the step writes) of every node
 //   phase_force     du = F/rho
 //   phase_collide   dE, collision, push
 // with the fields in device memory between them.
@@ -10,7 +10,7 @@
 // a node against 0.1 ns for the 608 bytes of populations.  The fused march
 // (fused.cuh) recomputes the moments and forces of every tile's ring, which
 // saves bytes that are free here and costs instructions that are not; it also
-// needs tiles to fill the chip.  Field traffic (14 values a node) is nothing
+// needs tiles to fill the chip.  Field traffic (13 values a node) is nothing
 // beside the arithmetic.  The per-node arithmetic is the march's
 // (node.cuh): the two forms agree bit for bit.  Measured, march -> phases, us
 // per step: D2Q9 128 x 128 125 -> 14.2, a row of 128 nodes 35 -> 12.7, D3Q19
@@ -34,8 +34,26 @@
 
 namespace lbm {
 
-// extra field planes of the phases, beyond F_COUNT (kernels.cuh)
-enum { X_E = 0, X_P = 1, X_COUNT = 2 };
+// E and P of a node wait for its collision in the buffer the step writes: the
+// pair of direction 0 stays at its node, so nothing but the node's own
+// collision writes it.  Only nodes the launch collides use it (the others'
+// pairs may be in place already, from another range of the same step).  A pair
+// of FP16 storage holds E alone; P follows from rho and T as it did before.
+__device__ __forceinline__ void put_scratch(Pop<float>* q, float E, float P) { q->v = make_float2(E, P); }
+__device__ __forceinline__ void put_scratch(Pop<double>* q, double E, double P) { q->v = make_double2(E, P); }
+__device__ __forceinline__ void put_scratch(Pop<__half>* q, float E, float) { q->v = __float_as_uint(E); }
+template <typename R> struct EnergyPressure {
+    R E, P;
+};
+__device__ __forceinline__ EnergyPressure<float> get_scratch(const Pop<float>* q, const KParams<float>&, float, float) {
+    return {q->v.x, q->v.y};
+}
+__device__ __forceinline__ EnergyPressure<double> get_scratch(const Pop<double>* q, const KParams<double>&, double, double) {
+    return {q->v.x, q->v.y};
+}
+__device__ __forceinline__ EnergyPressure<float> get_scratch(const Pop<__half>* q, const KParams<float>& p, float rho, float T) {
+    return {__uint_as_float(q->v), eos_pressure(p, rho, T)};
+}
 
 struct PhaseGeom {
     int plane_n, nm;       // nodes of a plane of the last axis, planes
@@ -63,7 +81,7 @@ template <int Q, typename S, typename R> struct Phase {
 };
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_moments_kernel(const S* src, R* fld, R* ext,
+__global__ void __launch_bounds__(128) phase_moments_kernel(const S* src, S* dst, R* fld,
                                                             const __grid_constant__ KParams<R> p,
                                                             PhaseGeom G, Counters* cnt) {
     using Math = NodeMath<Q, S, R>;
@@ -84,16 +102,11 @@ __global__ void __launch_bounds__(128) phase_moments_kernel(const S* src, R* fld
     if (Q == 19) fld[F_UZ * nn + n] = o.jm * inv;
     fld[F_T * nn + n] = T;
     fld[F_PHI * nn + n] = Math::phi_of(U);
-    ext[X_E * nn + n] = o.E;
-    ext[X_P * nn + n] = P;
-    const bool clamp = U >= R(0), bad = !(Math::positive(o.rho) && Math::positive(o.E));
-    if (clamp || bad) {   // counted once a step, with the plane's collision
-        const int m = n / G.plane_n;
-        if (m >= G.m_lo && m < G.m_hi) {
-            if (clamp) atomicAdd(&cnt->clamps, 1ull);
-            if (bad) atomicAdd(&cnt->bad, 1ull);
-        }
-    }
+    if (n < G.m_lo * G.plane_n || n >= G.m_hi * G.plane_n) return;
+    put_scratch(reinterpret_cast<Pop<S>*>(dst) + n, o.E, P);
+    // counted once a step, with the plane's collision
+    if (U >= R(0)) atomicAdd(&cnt->clamps, 1ull);
+    if (!(Math::positive(o.rho) && Math::positive(o.E))) atomicAdd(&cnt->bad, 1ull);
 }
 
 template <int Q, typename S, typename R>
@@ -120,7 +133,7 @@ __global__ void __launch_bounds__(128) phase_force_kernel(R* fld, const __grid_c
 }
 
 template <int Q, typename S, typename R>
-__global__ void __launch_bounds__(128) phase_collide_kernel(const S* src, S* dst, const R* fld, const R* ext,
+__global__ void __launch_bounds__(128) phase_collide_kernel(const S* src, S* dst, const R* fld,
                                                             const __grid_constant__ KParams<R> p, PhaseGeom G) {
     using Ph = Phase<Q, S, R>;
     using Math = NodeMath<Q, S, R>;
@@ -168,10 +181,11 @@ __global__ void __launch_bounds__(128) phase_collide_kernel(const S* src, S* dst
             }
         }
     }
-    const R dE = Math::energy_change(p, rho, T, ext[X_P * nn + n], ax, D);
-    const unsigned nbits = Store<S, R>::kStochastic ? node_bits(p.step, (unsigned)n) : 0u;
     Pop<S>* out = reinterpret_cast<Pop<S>*>(dst);
-    Math::collide(p, rho, ext[X_E * nn + n], u, dv, dE, [&](int k) { return f[k]; }, [&](int k, Two<R> v) {
+    const EnergyPressure<R> ep = get_scratch(out + n, p, rho, T);
+    const R dE = Math::energy_change(p, rho, T, ep.P, ax, D);
+    const unsigned nbits = Store<S, R>::kStochastic ? node_bits(p.step, (unsigned)n) : 0u;
+    Math::collide(p, rho, ep.E, u, dv, dE, [&](int k) { return f[k]; }, [&](int k, Two<R> v) {
         const unsigned t = Store<S, R>::kStochastic ? pair_word(nbits, k) : 0u;
         int to = n;
         bool bounce = false;
