@@ -21,7 +21,7 @@ struct lbm_handle {
     void* cnt = nullptr;        // lbm::Counters on the device
     double* partials = nullptr; // reduction scratch: block partials + 8 results
     double* staging = nullptr;  // (D + 3) planes of doubles for host transfers, allocated on demand
-    void* bounce = nullptr;     // pinned host buffer for small host outputs, allocated on demand
+    unsigned char* bounce = nullptr;   // host buffer the kernels write small host outputs to, allocated on demand
     void* coex = nullptr;       // coexistence table (arithmetic type) when p.latent != 0
     unsigned long long reported_bad = 0;
     long long steps = 0;

@@ -186,10 +186,30 @@ int be_output(lbm_handle* h, const lbm::Outputs& o, lbm::Counters* cnt_out) {
 }
 
 // Host outputs of at most this many bytes are written by the kernels straight
-// into a pinned buffer, with the counters, and copied from there by the host:
-// every copy from the device to pageable memory takes about 8 us, whatever its
-// size (a row of 128 nodes: four fields and the counters 80 us -> 35 us).
+// into a buffer of the handle in ordinary host memory, with the counters, and
+// copied from there by the host: every copy from the device to pageable memory
+// takes about 8 us, whatever its size (a row of 128 nodes: four fields and the
+// counters 80 us -> 35 us).  The GPU of a GB300 writes pageable memory through
+// the host's page tables as fast as pinned memory (4 KiB to 128 KiB: 10.1 to
+// 17.2 us against 10.3 to 17.3), and pinned memory would cost every handle 250
+// us to get and give back, more than all reads of a job that is read once.
 constexpr size_t kBounceBytes = 128 << 10;
+
+// the handle's buffer, allocated on first use; false where the device cannot
+// write it (the outputs then go through device memory)
+int ensure_bounce(lbm_handle* h, size_t bytes, bool& usable) {
+    usable = h->bounce != nullptr;
+    int direct = 0;
+    if (usable || cudaDeviceGetAttribute(&direct, cudaDevAttrPageableMemoryAccess, h->p.device) != cudaSuccess || !direct)
+        return LBM_OK;
+    h->bounce = new (std::nothrow) unsigned char[bytes]();   // zeroed: its pages are there
+    if (!h->bounce) {
+        set_error("output buffer allocation failed");
+        return LBM_ERR_OOM;
+    }
+    usable = true;
+    return LBM_OK;
+}
 
 // The output fields of the current state.
 int output_fields(lbm_handle* h, const lbm::Outputs& o, int mem) {
@@ -206,15 +226,15 @@ int output_fields(lbm_handle* h, const lbm::Outputs& o, int mem) {
         unsigned char* dev;
     } f[4] = {{o.rho, plane, nullptr}, {o.u, plane * h->D, nullptr}, {o.T, plane, nullptr}, {o.P, plane, nullptr}};
     const size_t total = plane * (size_t)(h->D + 3), counters = (sizeof(lbm::Counters) + 63) & ~(size_t)63;
-    const bool small = total <= kBounceBytes;
-    if (small && !h->bounce) {   // room for doubles, should the next call ask for them
+    bool small = total <= kBounceBytes;
+    if (small) {   // room for doubles, should the next call ask for them
         const size_t most = std::min(kBounceBytes, sizeof(double) * (size_t)(h->D + 3) * (size_t)h->nn);
-        if ((rc = cuda_error(cudaMallocHost(&h->bounce, counters + most), "output buffer allocation"))) return rc;
+        if ((rc = ensure_bounce(h, counters + most, small))) return rc;
     }
     // FP32 outputs of larger domains stage in the idle population buffer (at
     // least (d + 3) floats per node in every storage format)
     if (!small && !o.single && (rc = ensure_staging(h))) return rc;
-    unsigned char* at = small ? (unsigned char*)h->bounce + counters
+    unsigned char* at = small ? h->bounce + counters
                               : (unsigned char*)(o.single ? h->pop[h->cur ^ 1] : (void*)h->staging);
     for (Field& x : f) {
         if (x.dst) x.dev = at;
@@ -629,7 +649,7 @@ void lbm_destroy(lbm_handle* h) {
     cudaFree(h->slab);
     cudaFree(h->staging);
     cudaFree(h->coex);
-    cudaFreeHost(h->bounce);
+    delete[] h->bounce;
     delete h;
 }
 
