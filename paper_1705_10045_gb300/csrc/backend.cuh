@@ -14,6 +14,7 @@
 #include "kernels.cuh"
 #include "output.cuh"
 #include "phases.cuh"
+#include "plan.h"
 #include "rows.cuh"
 #include "strip.cuh"
 
@@ -47,8 +48,6 @@ template <typename R> KParams<R> make_kparams(const lbm_handle* h) {
 }
 
 inline unsigned grid_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
-
-constexpr int kSms = 152;   // SMs of a GB300
 
 // Launch a kernel that begins with griddepcontrol.wait as a programmatic
 // dependent of the stream's previous kernel: its CTAs are set up while that
@@ -100,103 +99,33 @@ template <int Q, typename S, typename R> struct Impl {
     static constexpr bool kF64 = std::is_same<S, double>::value;
     static constexpr bool kPhases = kF64 || Q == 19;
     static bool phases(const lbm_handle* h) { return kPhases && h->phases && h->fault_drop <= 0; }
+    static constexpr StepModel kModel = sizeof(S) == 2 ? kModelFp16 : kModelFp32;
+    static_assert(kF64 || Q == 9 || (kModel.tx == TX && kModel.ty == TY), "modelled tile");
     static bool wants_phases(const lbm_params& p) {
         if (kF64) return true;
         if (!kPhases) return false;
-        MarchGeom G;
-        G.na = p.nx;
-        G.nb = p.ny;
-        G.nm = p.nz;
-        double t, rows;
-        march_chunk(G, p.nz, t);
-        row_chunk(p, G, p.nz, rows);
-        const double nodes = (double)p.nx * p.ny * p.nz;
-        const double ns = 4.0 * 19 * sizeof(S) * nodes < 110e6 ? kPhaseNsL2 : kPhaseNs;   // both buffers stay in L2
-        return 4.5 + ns * 1e-3 * nodes < std::min(t, rows);
+        const MarchGeom G = {p.nx, p.ny, p.nz, 0, 0, p.nz};
+        return phase_time(kModel, G) < std::min(march_chunk(kModel, G, p.nz).t, row_chunk(kModel, G, p.nz, p.wall_x).t);
     }
     static int launches(const lbm_handle* h) {
         return h->p.step_kernel == LBM_STEP_THREE_LAUNCH || phases(h) ? 3 : 1;
     }
 
-    // D3Q19 in FP32 and FP16 storage has three forms of a step with the same
-    // bits, and takes the one with the smallest modelled time.  Measured us per
-    // step (march / row march / phases): FP32 32^3 33 / - / 7.4, 64^3 35 / 30 /
-    // 22.6, 80^3 54 / 42 / 51, 96^3 75 / 77 / 89, 128^3 160 / 150 / 202, 192^3 493
-    // / 478 / 662, 300^3 1996 / 1705 / -, 448 x 300 x 100 994 / 870 / -, 384 x 384 x
-    // 256 2545 / 2325 / -; FP16 64^3 33 / 24 / 19.4, 96^3 63 / 55 / 68, 128^3 140 /
-    // 124 / 152, 192^3 399 / 343 / 485, 384 x 384 x 256 2020 / 1710 / -.
-    //
-    // Phases: 4.5 us and kPhaseNs (kPhaseNsL2 where both buffers stay in L2) per
-    // node.
-    static constexpr double kPhaseNs = sizeof(S) == 2 ? 0.070 : 0.093, kPhaseNsL2 = sizeof(S) == 2 ? 0.057 : 0.072;
-    // March: planes per CTA, and its modelled time t.  A CTA takes about 4.5
-    // plane times beyond its chunk (ring planes, the first three planes'
-    // moments).  A plane takes kPlane1 us while an SM holds one CTA and kPlane2
-    // with two (64^3 in chunks of 8 with 128 CTAs, 128^3 in chunks of 32 with
-    // 256), 6 % more where CTAs of several waves run out of step; chunks stay
-    // below 65 planes so that neighbouring tiles keep sharing ring lines in L2.
-    // The chunk with the smallest modelled time avoids nearly empty last waves:
-    // FP32, two CTAs' worth of planes -> this: 128^3 195 -> 160 (5 -> 4 chunks),
-    // 160 x 128 x 96 188 -> 165, 192^3 569 -> 493.
-    static constexpr double kPlane1 = sizeof(S) == 2 ? 2.6 : 2.7, kPlane2 = sizeof(S) == 2 ? 3.85 : 4.4;
-    // Row march (rows.cuh): planes per CTA, and its modelled time t: one CTA per
-    // SM, (planes + 2.5) times kRowPlane us a wave.  0 where it does not run:
-    // walls on x, rows that are no multiple of 16 bytes.
+    // D2Q9 in FP32 and FP16 storage: a warp per strip of columns (strip.cuh)
+    static constexpr bool kStrips = Q == 9 && !kF64;
     static constexpr bool kRows = Q == 19 && !kF64;
-    static constexpr double kRowPlane = sizeof(S) == 2 ? 3.1 : 2.25;
-    static int row_chunk(const lbm_params& p, const MarchGeom& G, int len, double& t) {
-        int best = 0;
-        t = 1e30;
-        if constexpr (kRows) {
-            if (p.wall_x || G.na % (8 / (int)sizeof(S)) != 0) return 0;
-            const long long tiles = (long long)strip_count(G.na) * ((G.nb + RowShape<S>::TY - 1) / RowShape<S>::TY);
-            for (int n = (len + 63) / 64; n <= len; ++n) {
-                const int c = (len + n - 1) / n;
-                if ((len + c - 1) / c != n) continue;
-                const double tn = (c + 2.5) * kRowPlane * (double)((tiles * n + kSms - 1) / kSms);
-                if (tn < t) {
-                    t = tn;
-                    best = c;
-                }
-            }
-        }
-        return best;
-    }
 
-    // planes per CTA of the row march where it is modelled faster than the march, else 0
-    static int rows_instead(const lbm_params& p, const MarchGeom& G) {
-        double rows, march;
-        const int c = row_chunk(p, G, G.m_hi - G.m_lo, rows);
-        march_chunk(G, G.m_hi - G.m_lo, march);
-        return rows < march ? c : 0;
-    }
-
-    static int march_chunk(const MarchGeom& G, int len, double& t) {
-        const long long tiles = (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY);
-        const int few = (len + 63) / 64;   // chunks per column of tiles, at least
-        int best = len;
-        t = 1e30;
-        for (int n = few; n <= len; ++n) {
-            const int c = (len + n - 1) / n;
-            if ((len + c - 1) / c != n) continue;
-            const long long ctas = tiles * n, full = ctas / (2 * kSms), rest = ctas % (2 * kSms);
-            const double tn = (c + 4.5) * ((double)full * kPlane2 + (rest > kSms ? kPlane2 : (rest ? kPlane1 : 0.0))) *
-                              (full ? 1.06 : 1.0);
-            if (tn < t) {
-                t = tn;
-                best = c;
-            }
-            // four waves and more: the block scheduler evens out the last one
-            // (384 x 384 x 256: chunks of 64 2545 us, of 52 2597)
-            if (tiles * few >= 8 * kSms) break;
-        }
-        return best;
-    }
-
-    // planes [m_lo, m_hi) collided; m_hi < 0: the handle's own range
-    // (lbm_set_step_planes; all by default)
-    static MarchGeom geometry(const lbm_handle* h, int m_lo = 0, int m_hi = -1) {
-        MarchGeom G;
+    // How a step of planes [m_lo, m_hi) is launched, found once per call.
+    enum Form { kFormPhases, kFormStrips, kFormRows, kFormMarch, kFormFault };
+    struct Plan {
+        Form form;
+        MarchGeom G;     // chunk: of rows and march
+        int strip_rows;
+    };
+    // m_hi < 0: the handle's own range (lbm_set_step_planes; all by default)
+    static Plan plan(const lbm_handle* h, int m_lo = 0, int m_hi = -1) {
+        Plan s{};
+        MarchGeom& G = s.G;
         G.na = h->p.nx;
         G.nb = Q == 9 ? 1 : h->p.ny;
         G.nm = Q == 9 ? h->p.ny : h->p.nz;
@@ -207,31 +136,27 @@ template <int Q, typename S, typename R> struct Impl {
             G.m_lo = m_lo;
             G.m_hi = m_hi;
         }
-        double t;
-        G.chunk = march_chunk(G, G.m_hi - G.m_lo, t);
-        return G;
+        const int len = G.m_hi - G.m_lo;
+        if (h->fault_drop > 0) {   // fault-injection test hook (lbm_test_drop_handoff)
+            s.form = kFormFault;
+            G.chunk = std::min(kMaxChunk, len);   // long, so that the first CTA marches over the plane
+        } else if (phases(h)) {
+            s.form = kFormPhases;
+        } else if (kStrips) {
+            s.form = kFormStrips;
+            s.strip_rows = strip_rows(strip_count(G.na), len, kSms);
+        } else {
+            const Chunk march = march_chunk(kModel, G, len), rows = row_chunk(kModel, G, len, h->p.wall_x);
+            s.form = rows.t < march.t ? kFormRows : kFormMarch;
+            G.chunk = rows.t < march.t ? rows.planes : march.planes;
+        }
+        return s;
     }
 
     // name of the kernel of a step in one launch
     static const char* single_name(const lbm_handle* h) {
-        if (kStrips) return "strip_step_kernel";
-        return rows_instead(h->p, geometry(h)) > 0 ? "row_march_kernel" : "fused_step_kernel";
-    }
-
-    static void launch_fused(lbm_handle* h, const KParams<R>& kp) {
-        launch_fused_range(h, kp, geometry(h), (const S*)h->pop[h->cur], (S*)h->pop[h->cur ^ 1]);
-        h->cur ^= 1;
-    }
-
-    // D2Q9 in FP32 and FP16 storage: a warp per strip of columns (strip.cuh)
-    static constexpr bool kStrips = Q == 9 && !std::is_same<S, double>::value;
-
-    static StripGeom strip_geometry(const MarchGeom& G) {
-        StripGeom s;
-        s.na = G.na; s.nm = G.nm; s.m_lo = G.m_lo; s.m_hi = G.m_hi;
-        s.strips = strip_count(G.na);
-        s.chunk = strip_rows(s.strips, G.m_hi - G.m_lo, kSms);
-        return s;
+        const Form f = plan(h).form;
+        return f == kFormStrips ? "strip_step_kernel" : (f == kFormRows ? "row_march_kernel" : "fused_step_kernel");
     }
 
     // the step over the planes of G in three launches
@@ -263,49 +188,47 @@ template <int Q, typename S, typename R> struct Impl {
         if (j == 2) launch_after(phase_collide_kernel<Q, S, R>, grid, 128, 0, h->stream, src, dst, fld, kp, g);
     }
 
-    // the fused step over the planes of G, src -> dst (no buffer swap)
-    static void launch_fused_range(lbm_handle* h, const KParams<R>& kp, const MarchGeom& G, const S* src, S* dst) {
+    // the planned step, src -> dst (no buffer swap)
+    static void launch_fused(lbm_handle* h, const KParams<R>& kp, const Plan& s, const S* src, S* dst) {
         Counters* cnt = (Counters*)h->cnt;
-        if (h->fault_drop > 0) {   // fault-injection test hook (lbm_test_drop_handoff)
-            launch_fault(h, kp, G, src, dst);
-            return;
-        }
-        if constexpr (kPhases) {
-            if (kF64 || phases(h)) {
+        const MarchGeom& G = s.G;
+        const int len = G.m_hi - G.m_lo;
+        if (s.form == kFormPhases) {
+            if constexpr (kPhases)
                 for (int j = 0; j < 3; ++j) launch_phase(h, kp, G, src, dst, j);
-                return;
+        } else if (s.form == kFormStrips) {
+            if constexpr (kStrips) {
+                const StripGeom g = {G.na, G.nm, G.m_lo, G.m_hi, s.strip_rows, strip_count(G.na)};
+                const long long warps = (long long)g.strips * ((len + g.chunk - 1) / g.chunk);
+                auto kern = h->p.wall || h->p.wall_x ? strip_step_kernel<S, R, true> : strip_step_kernel<S, R, false>;
+                const size_t smem = kStripWarps * Strip<S, R, false>::kRingBytes;
+                allow_smem(kern, smem, h->fused_ready);
+                launch_after(kern, grid_for(warps, kStripWarps), 32 * kStripWarps, smem, h->stream, src, dst, kp, g, cnt);
             }
-        }
-        if constexpr (kF64) {
-            return;
-        } else if constexpr (kStrips) {
-            const StripGeom g = strip_geometry(G);
-            const long long warps = (long long)g.strips * ((g.m_hi - g.m_lo + g.chunk - 1) / g.chunk);
-            auto kern = h->p.wall || h->p.wall_x ? strip_step_kernel<S, R, true> : strip_step_kernel<S, R, false>;
-            const size_t smem = kStripWarps * Strip<S, R, false>::kRingBytes;
-            allow_smem(kern, smem, h->fused_ready);
-            launch_after(kern, grid_for(warps, kStripWarps), 32 * kStripWarps, smem, h->stream, src, dst, kp, g, cnt);
-        } else {
+        } else if (s.form == kFormRows) {
             if constexpr (kRows) {
-                MarchGeom g = G;
-                if ((g.chunk = rows_instead(h->p, G)) > 0) {
-                    using Sh = RowShape<S>;
-                    constexpr size_t smem = RowMarch<S, R, Sh::TY, Sh::AHEAD, true>::kBytes;
-                    auto kern = h->p.wall || h->p.wall_y ? row_march_kernel<S, R, true> : row_march_kernel<S, R, false>;
-                    allow_smem(kern, smem, h->rows_ready);
-                    launch_after(kern, dim3(strip_count(G.na), (G.nb + Sh::TY - 1) / Sh::TY,
-                                            (G.m_hi - G.m_lo + g.chunk - 1) / g.chunk),
-                                 32 * (Sh::TY + 4), smem, h->stream, src, dst, kp, g, cnt);
-                    return;
-                }
+                using Sh = RowShape<S>;
+                static_assert(Sh::TY == kModel.rows, "modelled tile");
+                constexpr size_t smem = RowMarch<S, R, Sh::TY, Sh::AHEAD, true>::kBytes;
+                auto kern = h->p.wall || h->p.wall_y ? row_march_kernel<S, R, true> : row_march_kernel<S, R, false>;
+                allow_smem(kern, smem, h->rows_ready);
+                launch_after(kern, dim3(strip_count(G.na), (G.nb + Sh::TY - 1) / Sh::TY, (len + G.chunk - 1) / G.chunk),
+                             32 * (Sh::TY + 4), smem, h->stream, src, dst, kp, G, cnt);
             }
+        } else {
             const size_t smem = FusedShape<TX, TY, SPLIT>::template smem_bytes<R>();
-            const bool xw = h->p.wall_x || (Q == 19 && h->p.wall_y);
-            auto kern = xw ? fused_step_kernel<Q, S, R, TX, TY, NP, true, SPLIT>
-                           : fused_step_kernel<Q, S, R, TX, TY, NP, false, SPLIT>;
-            allow_smem(kern, smem, h->fused_ready);
-            const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
-            kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, cnt);
+            const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (len + G.chunk - 1) / G.chunk);
+            if (s.form == kFormFault) {
+                auto kern = fused_step_fault_kernel<Q, S, R, TX, TY, NP, SPLIT>;
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, cnt, h->fault_drop - 1);
+            } else if constexpr (kRows) {
+                const bool xw = h->p.wall_x || h->p.wall_y;
+                auto kern = xw ? fused_step_kernel<Q, S, R, TX, TY, NP, true, SPLIT>
+                               : fused_step_kernel<Q, S, R, TX, TY, NP, false, SPLIT>;
+                allow_smem(kern, smem, h->fused_ready);
+                kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, cnt);
+            }
         }
     }
     // raise a kernel's shared-memory limit, once per handle
@@ -313,38 +236,27 @@ template <int Q, typename S, typename R> struct Impl {
         if (!ready) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         ready = true;
     }
-    // the march with the fault-injection hook; long chunks, so that the first
-    // CTA marches over the plane
-    static void launch_fault(lbm_handle* h, const KParams<R>& kp, MarchGeom G, const S* src, S* dst) {
-        G.chunk = std::min(64, G.m_hi - G.m_lo);
-        const size_t smem = FusedShape<TX, TY, SPLIT>::template smem_bytes<R>();
-        const dim3 grid((G.na + TX - 1) / TX, (G.nb + TY - 1) / TY, (G.m_hi - G.m_lo + G.chunk - 1) / G.chunk);
-        auto kern = fused_step_fault_kernel<Q, S, R, TX, TY, NP, SPLIT>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, TX * TY + NP, smem, h->stream>>>(src, dst, kp, G, (Counters*)h->cnt, h->fault_drop - 1);
-    }
-
     // planes [first, first + count) of the step lbm_step_begin opened: it has
     // already made the destination buffer current, so the source is the other
     static int step_range(lbm_handle* h, int first, int count) {
         KParams<R> kp = make_kparams<R>(h);
         kp.step = (unsigned)h->pending_step;
-        launch_fused_range(h, kp, geometry(h, first, first + count), (const S*)h->pop[h->cur ^ 1],
-                           (S*)h->pop[h->cur]);
+        launch_fused(h, kp, plan(h, first, first + count), (const S*)h->pop[h->cur ^ 1], (S*)h->pop[h->cur]);
         return cuda_error(cudaGetLastError(), "lbm_step_begin launch");
     }
 
     // launch j of one time step; the last launch of a step swaps the buffers
-    static void launch(lbm_handle* h, const KParams<R>& kp, int j) {
+    static void launch(lbm_handle* h, const KParams<R>& kp, const Plan& s, int j) {
         if (h->p.step_kernel != LBM_STEP_THREE_LAUNCH) {
-            if constexpr (kPhases) {
-                if (phases(h)) {
-                    launch_phase(h, kp, geometry(h), (const S*)h->pop[h->cur], (S*)h->pop[h->cur ^ 1], j);
-                    if (j == 2) h->cur ^= 1;
-                    return;
-                }
+            const S* src = (const S*)h->pop[h->cur];
+            S* dst = (S*)h->pop[h->cur ^ 1];
+            if (s.form == kFormPhases) {
+                if constexpr (kPhases) launch_phase(h, kp, s.G, src, dst, j);
+                if (j < 2) return;
+            } else {
+                launch_fused(h, kp, s, src, dst);
             }
-            launch_fused(h, kp);
+            h->cur ^= 1;
             return;
         }
         const unsigned g = grid_for(h->nn, 256);
@@ -362,9 +274,10 @@ template <int Q, typename S, typename R> struct Impl {
     static int step(lbm_handle* h, int n) {
         KParams<R> kp = make_kparams<R>(h);
         const int L = launches(h);
+        const Plan how = plan(h);
         for (int s = 0; s < n; ++s) {
             kp.step = (unsigned)(h->steps + s);
-            for (int j = 0; j < L; ++j) launch(h, kp, j);
+            for (int j = 0; j < L; ++j) launch(h, kp, how, j);
         }
         return cuda_error(cudaGetLastError(), "lbm_step launch");
     }
@@ -373,6 +286,7 @@ template <int Q, typename S, typename R> struct Impl {
     static int profile(lbm_handle* h, int n, double* ms, int cap) {
         KParams<R> kp = make_kparams<R>(h);
         const int L = launches(h);
+        const Plan how = plan(h);
         cudaEvent_t ev[6];
         for (int e = 0; e < 2 * L; ++e)
             if (int rc = cuda_error(cudaEventCreate(&ev[e]), "event create")) return rc;
@@ -382,7 +296,7 @@ template <int Q, typename S, typename R> struct Impl {
             kp.step = (unsigned)(h->steps + s);
             for (int j = 0; j < L; ++j) {
                 cudaEventRecord(ev[2 * j], h->stream);
-                launch(h, kp, j);
+                launch(h, kp, how, j);
                 cudaEventRecord(ev[2 * j + 1], h->stream);
             }
             rc = cuda_error(cudaEventSynchronize(ev[2 * L - 1]), "profile synchronize");
@@ -448,7 +362,7 @@ template <int Q, typename S, typename R> struct Impl {
             long long items = 0;
             for (const MarchGeom& G : in)
                 items += (long long)((G.na + TX - 1) / TX) * ((G.nb + TY - 1) / TY) * ((G.nm + c - 1) / c);
-            const double t = (c + 4.5) * (items > kSms ? kPlane2 : kPlane1) *
+            const double t = (c + 4.5) * (items > kSms ? kModel.plane2 : kModel.plane1) *
                              std::max(1.0, (double)items / (2.0 * kSms));
             if (t <= best_t) {
                 best_t = t;

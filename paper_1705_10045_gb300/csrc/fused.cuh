@@ -45,6 +45,7 @@
 #pragma once
 
 #include "node.cuh"
+#include "plan.h"
 #include "strip.cuh"
 
 namespace lbm {
@@ -93,14 +94,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity
     } while (clock64() - t0 < 1000000000ll);
     return false;
 }
-
-// Geometry of the march: na x nb tile plane (nb = 1 for D2Q9), nm planes.
-struct MarchGeom {
-    int na, nb, nm;
-    int chunk;        // planes per CTA along the march axis
-    int m_lo, m_hi;   // planes whose collision the launch runs (the moment and
-                      // force stages reach two and one planes beyond them)
-};
 
 // Plane buffers: Phi for 3 planes, rho/u/T for 5 planes, du for 4 planes
 // (the consumer trails the producer by three planes).  SPLIT: the consumers

@@ -27,15 +27,9 @@
 #pragma once
 
 #include "node.cuh"
+#include "plan.h"
 
 namespace lbm {
-
-struct StripGeom {
-    int na, nm;       // columns (x) and rows (y) of the domain
-    int m_lo, m_hi;   // rows the launch collides
-    int chunk;        // rows per work item
-    int strips;       // ceil(na / kCols)
-};
 
 // asynchronous copy of one stored pair into shared memory
 template <typename S> __device__ __forceinline__ void copy_async(Pop<S>* to, const Pop<S>* from) {
@@ -46,9 +40,6 @@ template <typename S> __device__ __forceinline__ void copy_async(Pop<S>* to, con
 
 // WALL: the domain has walls on x or y (the other instance is periodic and
 // carries no trace of them).
-constexpr int kStripCols = 28;   // columns a warp collides
-__host__ __device__ inline int strip_count(int na) { return (na + kStripCols - 1) / kStripCols; }
-
 template <typename S, typename R, bool WALL> struct Strip {
     static constexpr int Q = 9;
     static constexpr int kCols = kStripCols;
@@ -237,38 +228,6 @@ template <typename S, typename R, bool WALL> struct Strip {
         }
     }
 };
-
-// Warps per CTA: strips of one CTA are neighbours in x, so the ring columns
-// they share come from L1.
-constexpr int kStripWarps = 4;
-constexpr int kStripCtas = 4;   // CTAs per SM the kernel is compiled for (128 registers)
-
-// Rows per warp.  More rows per warp repeat fewer ring rows (the four extra
-// rows of a warp cost about 1.25 full rows); fewer rows give more warps, which
-// a small domain needs to fill 152 SMs.  The time of a launch is modelled as
-// its waves of CTAs, each (rows + 1.25) times the time of one row with w warps
-// per SM, 0.3 + 0.072 w us (measured: 0.58 us with 4, 0.85 with 8, 1.45 with
-// 16), and the row count with the smallest modelled time is taken.  Measured
-// us per step around the choice: 128 x 128 2 rows 3.7, 4 rows 5.0, 8 rows
-// 7.5; 512 x 512 4 rows 8.4, 8 rows 9.6, 16 rows 12.7; 1000 x 1000 8 rows
-// 29.3, 16 rows 27.8, 32 rows 32.8; 8192 x 4608 32 rows 903, 64 rows 895.
-inline int strip_rows(int strips, int len, int sms) {
-    int best = 1;
-    double best_t = 1e30;
-    for (int c : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 40, 48, 64}) {
-        if (c > len && c > 1) break;
-        const long long warps = (long long)strips * ((len + c - 1) / c);
-        const long long ctas = (warps + kStripWarps - 1) / kStripWarps;
-        const long long full = ctas / ((long long)kStripCtas * sms), rest = ctas % ((long long)kStripCtas * sms);
-        auto row = [&](long long per_sm) { return 0.3 + 0.072 * (double)(per_sm * kStripWarps); };
-        const double t = (c + 1.25) * ((double)full * row(kStripCtas) + (rest ? row((rest + sms - 1) / sms) : 0.0));
-        if (t < best_t) {
-            best_t = t;
-            best = c;
-        }
-    }
-    return best;
-}
 
 template <typename S, typename R, bool WALL>
 __global__ void __launch_bounds__(32 * kStripWarps, kStripCtas)
