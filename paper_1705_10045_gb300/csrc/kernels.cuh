@@ -287,6 +287,19 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// The sum of a few FP32 values as s + c + d, in FP32 arithmetic: two levels of
+// exact additions (Knuth's two-sum) and the rest in d, whose own rounding lies
+// below 2^-70 of the largest value.
+struct Expansion {
+    float s = 0.f, c = 0.f, d = 0.f;
+    __device__ static float two_sum(float& a, float b) {   // a += b; what the rounding left out
+        const float t = a + b, z = t - a, e = (a - (t - z)) + (b - z);
+        a = t;
+        return e;
+    }
+    __device__ void add(float v) { d += two_sum(c, two_sum(s, v)); }
+};
+
 // FP32 to FP64 in integer instructions for normal values (the conversion
 // instruction runs at the FP64 rate: two lanes per clock and SM)
 __device__ __forceinline__ double widen(double v) { return v; }
@@ -298,7 +311,8 @@ __device__ __forceinline__ double widen(float v) {
 
 // Blocks of a reduction over n nodes: at least four nodes per thread, so that
 // the FP64 block tails stay a minority, and at most one wave of three blocks
-// per SM (934 us on the pool-boiling domain; four 945, five 997, six 1024).
+// per SM (with groups in plain FP64 934 us on the pool-boiling domain; four
+// 945, five 997, six 1024).
 constexpr int kReduceCtas = 3;
 inline int reduce_blocks(long long n) {
     const long long per = 4 * kReduceThreads, b = (n + per - 1) / per, most = 152 * kReduceCtas;
@@ -312,12 +326,14 @@ inline int reduce_blocks(long long n) {
 // Bound by the FP64 pipe before memory: five Kahan additions a node are 20
 // FP64 instructions, at two lanes per clock and SM 1.3 ms for 37.7 M nodes,
 // where the populations stream in 0.85 ms.  So moments formed in FP32 are
-// first added up over kGroup nodes in plain FP64 (exact unless their
-// magnitudes spread over 2^26: 24-bit values in a 53-bit sum) and the group
-// sum enters the compensated one: 7.5 FP64 instructions a node.  FP64 moments
-// enter one by one.  Whole diagnostics call, before -> now: 384 x 384 x 256
-// D3Q19 FP32 2326 -> 934 us, FP16 2128 -> 912, 8192 x 4608 D2Q9 1760 -> 737,
-// 512 x 512 234 -> 48.
+// first added up over kGroup nodes in FP32 expansions, exactly for all that a
+// double holds, and the three parts enter the compensated sum: 7.5 FP64
+// instructions a node.  A group whose sum leaves the range of FP32 (or holds
+// an infinity or NaN) enters it node by node, as FP64 moments do.  Whole
+// diagnostics call, node by node -> this: 384 x 384 x 256 D3Q19 FP32 2309 -> 896
+// us, FP16 2107 -> 784, 8192 x 4608 D2Q9 1743 -> 610, 512 x 512 216 -> 41.
+// (Groups added up in plain FP64 lost what lies 2^-53 below a group's largest
+// value and were no faster: 916, 904, 729, 37.)
 template <int Q, typename S, typename R, bool PAIRS = true>
 __global__ void __launch_bounds__(kReduceThreads, kReduceCtas) reduce_kernel(const S* __restrict__ pop, long long nn, long long i0,
                                                                 long long n, KParams<R> p,
@@ -325,19 +341,41 @@ __global__ void __launch_bounds__(kReduceThreads, kReduceCtas) reduce_kernel(con
     constexpr int kGroup = sizeof(R) == 4 ? 8 : 1;
     Kahan acc[kSums];
     const long long stride = (long long)gridDim.x * blockDim.x;
+    auto moments = [&](long long at, R* m) {
+        node_moments<Q, S, R, PAIRS>(pop, nn, i0 + at, p, m[0], m[1], m[2], m[3], m[4]);
+    };
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kGroup * stride) {
-        double g[kSums];
+        R m[kSums];
+        bool summed = false;
+        if constexpr (kGroup > 1) {
+            Expansion g[kSums];
 #pragma unroll 1
-        for (int j = 0; j < kGroup; ++j) {
-            const long long at = i + j * stride;
-            if (at >= n) break;
-            R m[kSums];
-            node_moments<Q, S, R, PAIRS>(pop, nn, i0 + at, p, m[0], m[1], m[2], m[3], m[4]);
+            for (int j = 0; j < kGroup && i + j * stride < n; ++j) {
+                moments(i + j * stride, m);
 #pragma unroll
-            for (int q = 0; q < kSums; ++q) g[q] = j == 0 ? widen(m[q]) : g[q] + widen(m[q]);
+                for (int q = 0; q < kSums; ++q) g[q].add(m[q]);
+            }
+            float rest = 0.f;   // NaN unless every part is finite
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) rest += (g[q].s - g[q].s) + (g[q].c - g[q].c) + (g[q].d - g[q].d);
+            summed = rest == 0.f;
+            if (summed) {
+#pragma unroll
+                for (int q = 0; q < kSums; ++q) {
+                    acc[q].add(widen(g[q].s));
+                    acc[q].add(widen(g[q].c));
+                    acc[q].add(widen(g[q].d));
+                }
+            }
         }
+        if (!summed) {
+#pragma unroll 1
+            for (int j = 0; j < kGroup && i + j * stride < n; ++j) {
+                moments(i + j * stride, m);
 #pragma unroll
-        for (int q = 0; q < kSums; ++q) acc[q].add(g[q]);
+                for (int q = 0; q < kSums; ++q) acc[q].add((double)m[q]);
+            }
+        }
     }
     __shared__ double sh[kSums][kReduceThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
