@@ -254,7 +254,9 @@ int lbm_batch_add(lbm_batch* b, const lbm_params* p, const double* rho, const do
 /* Destroy a domain and free its slot (synchronising). */
 int lbm_batch_remove(lbm_batch* b, int id);
 
-/* Enqueue n step launches; every domain takes min(n, budget) steps. */
+/* Enqueue n steps; every domain takes min(n, budget) of them.  When a single
+ * domain has a budget it takes lbm_step's launches, with the same result.
+ * Refused (LBM_ERR_CUDA) while the batch's stream is being captured. */
 int lbm_batch_step(lbm_batch* b, int n);
 
 /* Steps a domain has taken since its initialisation and steps left in its budget. */

@@ -297,6 +297,13 @@ int lbm_batch_step(lbm_batch* b, int n) {
     }
     if (n == 0) return LBM_OK;
     cudaSetDevice(b->common.device);
+    // budgets and buffer indices live on the host, where a replayed graph would not move them
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (int rc = cuda_error(cudaStreamIsCapturing(b->stream, &capturing), "batch stream")) return rc;
+    if (capturing != cudaStreamCaptureStatusNone) {
+        set_error("lbm_batch_step: the batch's stream is being captured");
+        return LBM_ERR_CUDA;
+    }
     if (const int only = only_active(b); only >= 0 && b->fault_item < 0) return step_alone(b, only, n);
     if (b->dirty || table_set(b, false) != b->in_table)
         if (int rc = rebuild(b)) return rc;
