@@ -72,7 +72,8 @@ def _fields():
     return W.pool_boiling_3d(nx=NX, ny=NY, nz=NZ, T=0.8, depth=DEPTH, noise=1e-4, seed=3)
 
 
-KERNEL_SOURCES = ("rows.cuh", "strip.cuh", "fused.cuh", "node.cuh", "kernels.cuh", "lattice.cuh", "backend.cuh")
+KERNEL_SOURCES = ("rows.cuh", "strip.cuh", "fused.cuh", "phases.cuh", "node.cuh", "kernels.cuh", "lattice.cuh", "plan.h",
+                  "backend.cuh")
 TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "row_march_kernel_d3q19_fp32.md")
 
 

@@ -70,9 +70,9 @@ void launch_after(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cu
 
 // CTA shape of the fused kernel: a TX x TY tile of consumer threads plus NP
 // producer threads.  D3Q19 uses 32 x 8 nodes with 128 producers (two CTAs per
-// SM) in FP32/FP16 and 256 producers in FP64.  D2Q9 uses rows of 128 nodes
-// with 160 producers: one producer per node of the 132-node ring row, so the
-// moments of a row take a single round of loads.
+// SM) in FP32/FP16.  FP64 (256 producers on D3Q19) and D2Q9 (rows of 128 nodes
+// with 160 producers, one per node of the 132-node ring row) run it in its
+// fault-injection form only.
 // SPLIT: the consumers form the moments of their own nodes and the producers
 // only those of the ring's border (fused_tile)
 template <int Q, typename R> struct FusedTile;
@@ -345,6 +345,11 @@ template <int Q, typename S, typename R> struct Impl {
     // and only few or small domains need shorter ones to fill the chip.
     // Measured FP32, 64 planes -> this: 126^3 + 80^3 315 -> 215 us, four of 64^3
     // 259 -> 83, 33^3 + 46^3 + 63^3 243 -> 49, eight of 33..126 480 (64 planes).
+    // FP64, whose items are bound by arithmetic, follows the same lengths: D2Q9
+    // (march in items of 64 rows -> strips) 24 of 64..512 2389 -> 1571 us, 6 of
+    // 64..200 722 -> 130, 2 of 1000 2142 -> 1225; D3Q19 (64 planes -> this) four
+    // of 90 x 75 x 67 2837 -> 2422, 33^3 + 46^3 + 63^3 2771 -> 730, 126^3 + 80^3
+    // 3746 -> 3230.
     static int batch_chunk(const lbm_batch* b) {
         std::vector<MarchGeom> in;
         for (size_t d = 0; d < b->doms.size(); ++d)

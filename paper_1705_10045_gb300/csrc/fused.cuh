@@ -26,10 +26,10 @@
 // before F, and F before the next M, inside the producer warps.  Ring nodes
 // are recomputed by neighbouring CTAs from L2 rather than exchanged.  D2Q9
 // runs the same code as a lattice with one y node: its lattice y axis is the
-// march axis and its tile is TX x 1 (FP64 without memory for its phases, and
-// the fault-injection form; D2Q9 otherwise steps strips, strip.cuh).  Batches
-// of D3Q19 domains run it, and the single domains for which backend.cuh
-// models it faster than rows.cuh and phases.cuh.
+// march axis and its tile is TX x 1 (the fault-injection form only; D2Q9
+// otherwise steps strips, strip.cuh, or phases).  Batches of D3Q19 domains run
+// it, and the single FP32 and FP16 domains for which it is modelled faster
+// than rows.cuh and phases.cuh (plan.h).
 //
 // Index arithmetic is kept out of the inner loops: the wrapped ring
 // coordinates of a CTA are tabulated once in shared memory, buffer slots come
@@ -278,10 +278,12 @@ template <int Q, typename S, typename R, int TX, int TY, bool COH = false, bool 
         // each half is widened where it is used.
         const int n = c * plane_n + n_ab;
         Pop<S> w[Q];
+        const S* q = src + 2 * (size_t)n;
 #pragma unroll
-        { const S* q = src + 2 * (size_t)n;
-#pragma unroll
-        for (int k = 0; k < Q; ++k) { w[k] = load_pop<COH, kUseLast>(q, 0); q += 2 * nn; } }
+        for (int k = 0; k < Q; ++k) {
+            w[k] = load_pop<COH, kUseLast>(q, 0);
+            q += 2 * nn;
+        }
         const int sr = sl.rut, sd = sl.du();
         const R rho = rut(sr, 0, fc), T = rut(sr, 4, fc);
         const R u[3] = {rut(sr, 1, fc), rut(sr, 2, fc), rut(sr, 3, fc)};

@@ -58,7 +58,6 @@ struct lbm_batch {
     int variant = 0;                    // CTA shape (see lbm_batch_variants)
     void* d_sched = nullptr;            // lbm::BatchSched + done[descs_cap] + aborted[descs_cap]
     int* h_steps = nullptr;             // pinned staging of the request's step count
-    int sched_steps = 0;                // step count of the current request (host copy)
     int grid = 0;                       // persistent CTAs of the current shape
     bool xw = false;                    // some domain has walls that the kernel has to know of
     int fault_item = -1;                // lbm_batch_test_drop_item hook: item of step 0, -1 = off

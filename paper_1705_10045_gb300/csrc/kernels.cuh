@@ -12,6 +12,7 @@
 #pragma once
 
 #include "lattice.cuh"
+#include "plan.h"
 
 namespace lbm {
 
@@ -262,11 +263,11 @@ __global__ void __launch_bounds__(256) init_kernel(S* __restrict__ pop, const do
 
 // ---------------------------------------------------------------------------
 // Conservation sums in FP64 with Kahan compensation.  Each thread walks a
-// fixed strided set of nodes, blocks combine in a fixed shuffle tree and one
-// more block sums the block partials in a fixed order: bitwise reproducible
+// fixed strided set of nodes, blocks combine in a fixed shuffle tree and a
+// warp per sum adds the block partials in a fixed order: bitwise reproducible
 // for a given number of nodes.
 
-constexpr int kReduceBlocks = 1024;   // most blocks (and block partials) of a reduction
+constexpr int kReduceBlocks = 1024;   // block partials the scratch of a reduction holds (40,960 bytes, include/lbm.h)
 constexpr int kReduceThreads = 256;
 constexpr int kSums = 5;   // mass, momentum x, y, z, energy
 
@@ -314,8 +315,9 @@ __device__ __forceinline__ double widen(float v) {
 // per SM (with groups in plain FP64 934 us on the pool-boiling domain; four
 // 945, five 997, six 1024).
 constexpr int kReduceCtas = 3;
+static_assert(kSms * kReduceCtas <= kReduceBlocks, "reduction scratch");
 inline int reduce_blocks(long long n) {
-    const long long per = 4 * kReduceThreads, b = (n + per - 1) / per, most = 152 * kReduceCtas;
+    const long long per = 4 * kReduceThreads, b = (n + per - 1) / per, most = kSms * kReduceCtas;
     return (int)(b < 1 ? 1 : (b > most ? most : b));
 }
 

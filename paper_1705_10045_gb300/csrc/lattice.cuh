@@ -117,13 +117,14 @@ __host__ __device__ __forceinline__ size_t pair_index(int k, long long nn, long 
 template <typename S, typename R> struct Store;
 // load: one value at element index i (the set-major checkpoint layout).
 // load2 / store2: the pair (N_k, g_k) at pair index i in one access (shifts
-// sN, sG; random word t of the FP16 rounding).  load2_keep: a first read
-// of lines the same SM reads again soon (L2 evict-last where it pays).
-// load2_last: the read of a value's last use on this SM (the fused step's
-// consumer reload); L1::no_allocate leaves L1 to the lines the moment stage
-// will still reuse.  The _coh forms skip the non-coherent path, for data
-// other CTAs of the same launch wrote (read after an acquire of their
-// release).
+// sN, sG; random word t of the FP16 rounding).  load2_keep (FP32): a first
+// read of lines the same SM reads again soon (L2 evict-last).  load2_last: the
+// read of a value's last use on this SM (the fused step's consumer reload);
+// L1::no_allocate leaves L1 to the lines the moment stage will still reuse.
+// The _coh forms skip the non-coherent path, for data that is written while
+// the kernel is resident: by other CTAs of the same launch (read after an
+// acquire of their release), or by the launch before it (read behind
+// griddepcontrol.wait).  FP16 pairs move as words (word, word_last, _coh).
 
 template <> struct Store<double, double> {
     static constexpr bool kStochastic = false, kShifted = false;
@@ -132,9 +133,6 @@ template <> struct Store<double, double> {
         const double2 v = __ldg(reinterpret_cast<const double2*>(p) + i);
         a = v.x;
         b = v.y;
-    }
-    __device__ static void load2_keep(const double* p, size_t i, double sN, double sG, double& a, double& b) {
-        load2(p, i, sN, sG, a, b);
     }
     __device__ static void load2_last(const double* p, size_t i, double, double, double& a, double& b) {
         asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "l"(p + 2 * i));
@@ -219,18 +217,6 @@ template <> struct Store<__half, float> {
     }
     __device__ static void load2(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
         unpack(word(p, i), sN, sG, a, b);
-    }
-    __device__ static void load2_keep(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
-        load2(p, i, sN, sG, a, b);
-    }
-    __device__ static void load2_last(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
-        unpack(word_last(p, i), sN, sG, a, b);
-    }
-    __device__ static void load2_coh(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
-        unpack(word_coh(p, i), sN, sG, a, b);
-    }
-    __device__ static void load2_last_coh(const __half* p, size_t i, float sN, float sG, float& a, float& b) {
-        unpack(word_last_coh(p, i), sN, sG, a, b);
     }
     // the halves of a pair word widened, and sums with one half rounded once in
     // FP32 (mixed-precision add / sub: a half widens to FP32 exactly, so these

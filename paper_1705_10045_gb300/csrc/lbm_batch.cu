@@ -134,7 +134,6 @@ int upload_descs(lbm_batch* b, long long n) {
     if (b->common.storage == LBM_STORE_FP64) stage_descs<double>(b, n);
     else stage_descs<float>(b, n);
     *b->h_steps = (int)n;
-    b->sched_steps = (int)n;
     if (int rc = cuda_error(cudaMemcpyAsync(b->d_sched, b->h_steps, sizeof(int), cudaMemcpyHostToDevice, b->stream),
                             "batch step count copy"))
         return rc;

@@ -128,7 +128,7 @@ template <> struct Pop<__half> {
 };
 
 // The pair at pair index i of q.  COH: coherent loads, for data other CTAs of
-// the same launch wrote.  KEEP: a first read of lines the same SM reads again
+// the same launch or the launch before it wrote while this one was resident.  KEEP: a first read of lines the same SM reads again
 // soon (L2 evict-last where it pays).  LAST: the last use of the line on this
 // SM (not allocated in L1).
 enum LoadUse { kUse, kUseKeep, kUseLast };

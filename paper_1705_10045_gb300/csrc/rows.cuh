@@ -259,7 +259,8 @@ template <typename S, typename R, int TY, int AHEAD, bool WALL> struct RowMarch 
 };
 
 // Rows a CTA collides and planes loaded ahead: what 227 KB hold with two planes
-// ahead.  384 x 384 x 256, us per step: FP32 9 rows 2361, 8 rows 2418, 7 rows
+// ahead.  384 x 384 x 256 in chunks of 64 planes (the planned chunks are faster,
+// see above), us per step: FP32 9 rows 2361, 8 rows 2418, 7 rows
 // 2560, 6 rows with three planes ahead 2684, 10 rows with one 3470; FP16 16
 // rows 1830, 14 rows 2001, 18 rows 2671 (registers), 12 rows with three ahead
 // 1905.
