@@ -217,9 +217,9 @@ void lbm_destroy(lbm_handle* h);
 
 /* ---------------------------------------------------------------------------
  * Batches: many independent domains (different sizes, same lattice and
- * storage) advanced together.  lbm_batch_step(n) is one persistent kernel
- * launch that covers every step of every domain through a table of
- * (domain, tile, chunk) work items: CTAs take (step, item) work in order from
+ * storage) advanced together.  lbm_batch_step(n) of several stepping domains is
+ * one persistent kernel launch that covers every step of every domain through
+ * a table of (domain, tile, chunk) work items: CTAs take (step, item) work in order from
  * a counter, and an item of step s of a domain starts once every item of that
  * domain has finished step s - 1 (per-domain completion counters in device
  * memory, waits bounded to about half a second, then LBM_ERR_TIMEOUT on that

@@ -37,8 +37,8 @@ struct lbm_handle {
 };
 
 // Many domains advanced together (lbm_batch_*): every domain is an
-// lbm_handle; one persistent launch per request covers all of them and all
-// steps through a work table.
+// lbm_handle; one persistent launch per request covers all that step and all
+// steps through a work table (a domain that steps alone takes its own launches).
 struct lbm_batch {
     lbm_params common;
     int Q = 0;

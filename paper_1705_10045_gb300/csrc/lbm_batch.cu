@@ -2,7 +2,8 @@
 //
 // Every domain is an ordinary lbm_handle (own population buffers, counters
 // and moments scratch), created on the batch's stream.  One persistent launch
-// per request covers every step of every domain through a table of work
+// per request of several stepping domains (a single one takes its own launches,
+// step_alone) covers every step of every domain through a table of work
 // items (domain, tile, chunk); each domain's descriptor in device memory
 // holds its pointers, parameters, the buffer holding its state and the steps
 // it still takes in the request.  Inside the launch, per-domain completion
@@ -156,7 +157,7 @@ int only_active(const lbm_batch* b) {
 // A request in which one domain steps takes the single-domain step, whose
 // launches fit the domain (in phases where that is faster) and need no
 // completion counters: the same bits, FP32 126^3 300 -> 181 us a step (178
-// with the best chunk of the persistent launch), 64^3 260 -> 24.
+// with the best chunk of the persistent launch), 64^3 260 -> 22.
 int step_alone(lbm_batch* b, int d, int n) {
     lbm_handle* h = b->doms[d];
     const int m = (int)std::min<long long>(b->budget[d], n);

@@ -49,9 +49,9 @@ template <typename F> inline void each_chunk(int len, const F& f) {
 // D3Q19 in FP32 and FP16 storage has three forms of a step with the same
 // bits, and takes the one with the smallest modelled time.  Measured us per
 // step (march / row march / phases): FP32 32^3 33 / - / 7.4, 64^3 35 / 30 /
-// 22.6, 80^3 54 / 42 / 51, 96^3 75 / 77 / 89, 128^3 160 / 150 / 202, 192^3 493
+// 21.9, 80^3 54 / 42 / 51, 96^3 75 / 77 / 89, 128^3 160 / 150 / 202, 192^3 493
 // / 478 / 662, 300^3 1996 / 1705 / -, 448 x 300 x 100 994 / 870 / -, 384 x 384 x
-// 256 2545 / 2325 / -; FP16 64^3 33 / 24 / 19.4, 96^3 63 / 55 / 68, 128^3 140 /
+// 256 2545 / 2325 / -; FP16 64^3 33 / 24 / 18.9, 96^3 63 / 55 / 68, 128^3 140 /
 // 124 / 152, 192^3 399 / 343 / 485, 384 x 384 x 256 2020 / 1710 / -.
 struct StepModel {
     // phases: 4.5 us and ns per node (ns_l2 where both buffers stay in L2)
